@@ -252,8 +252,8 @@ size_t q0_partial_count(const int mesh[3], double beta, const double *lattice);
 // ------------------------------------------------------------ kernels (stage 1, k_stage1.cu)
 template <typename R>
 void launch_thetapsi(const double2 *d_theta, const int dlo[3], const int ddim[3], const int tlo[3],
-                     const int tdim[3], const double2 *d_c, const int *d_G, int nb, int npw,
-                     typename C2<R>::T *d_out, cudaStream_t st);
+                     const int tdim[3], const int *d_klist, int nklist, const double2 *d_c, const int *d_G, int nb,
+                     int npw, typename C2<R>::T *d_out, cudaStream_t st);
 template <typename R>
 void launch_bmat(const double2 *d_A, const double *d_R, const double *d_T, const double *d_gaunt,
                  int n_atoms, int lmax, int Lmax, int P, int nb, int use_T, typename C2<R>::T *d_B,
@@ -291,7 +291,10 @@ struct ZGemmBatch {         // C = op(A) * B, complex double, K = K1 * K2
     int M, N, K1, K2;
     long long sAi, sAk2, sAk1, sBk2, sBk1, sBj, sCi, sCj;
     int conjA;
+    int upper;              // apply only the upper triangle of A, half its diagonal (M = K2, K1 = 1)
+    int herm;               // C is Hermitian: compute its upper triangle, mirror the rest
 };
+int zgemm64_tile(int M, int N, long long nbatch);   // tile edge launch_zgemm64 takes for these sizes
 void launch_zgemm64(const ZGemmBatch *d_b, int nbatch, int maxM, int maxN, cudaStream_t st);
 void launch_block64(const QDesc *d_q, int nq, const double2 *const *d_VB, const double2 *d_Z, double2 *d_Y,
                     long long RSc, int nch, int P, int N0, long long maxcols, cudaStream_t st);
@@ -398,7 +401,7 @@ int zmt_tc_run_batch(hfx_ctx *ctx, const ZmtPlan &zs, const ZmtBatch &zb, const 
 // ------------------------------------------------------------ kernels (finish, k_finish.cu)
 void launch_reduce_pairs(const PairDesc *d_pairs, const int *d_kstart, const int *d_klist_pairs, int nk_in_batch,
                          const int *d_klist, const double *d_praw, const long long *d_praw_off, int NB, int raw_format,
-                         int real_part, double2 *const *d_vacc, const int *d_nb_k, int nb_max, cudaStream_t st);
+                         int nsplit, int real_part, double2 *const *d_vacc, const int *d_nb_k, int nb_max, cudaStream_t st);
 // V = -(1/N_k) Vacc - q->0 term (+ the k.p term d_kp[k] if d_kp is non-null), and E_x.
 void launch_finish(double2 *const *d_vacc, double2 *const *d_V, const int *d_nb_k, const int *d_no_k, int nk,
                    int nb_max, double inv_nk, double q0b, int q0_on, double2 *const *d_kp, double *d_Ex,

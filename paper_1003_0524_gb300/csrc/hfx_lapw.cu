@@ -96,17 +96,17 @@ int hfx_lapw_transform_all(hfx_ctx *ctx, hfx_stats *st) {
         ZGemmBatch &a = g1[ik];
         a.A = k.d_c; a.B = ctx->d_S[ik]; a.C = B;
         a.M = nb; a.N = np; a.K1 = 1; a.K2 = np;
-        a.sAi = np; a.sAk1 = 0; a.sAk2 = 1; a.sBk1 = 0; a.sBk2 = np; a.sBj = 1; a.sCi = np; a.sCj = 1; a.conjA = 1;
+        a.sAi = np; a.sAk1 = 0; a.sAk2 = 1; a.sBk1 = 0; a.sBk2 = np; a.sBj = 1; a.sCi = np; a.sCj = 1; a.conjA = 1; a.upper = 0; a.herm = 0;
         // W[n][G'] = sum_n' V[n][n'] B[n'][G']
         ZGemmBatch &b = g2[ik];
         b.A = ctx->d_V[ik]; b.B = B; b.C = W;
         b.M = nb; b.N = np; b.K1 = 1; b.K2 = nb;
-        b.sAi = nb; b.sAk1 = 0; b.sAk2 = 1; b.sBk1 = 0; b.sBk2 = np; b.sBj = 1; b.sCi = np; b.sCj = 1; b.conjA = 0;
+        b.sAi = nb; b.sAk1 = 0; b.sAk2 = 1; b.sBk1 = 0; b.sBk2 = np; b.sBj = 1; b.sCi = np; b.sCj = 1; b.conjA = 0; b.upper = 0; b.herm = 0;
         // V_GG'[G][G'] = sum_n conj(B[n][G]) W[n][G']
         ZGemmBatch &d = g3[ik];
         d.A = B; d.B = W; d.C = Vg;
         d.M = np; d.N = np; d.K1 = 1; d.K2 = nb;
-        d.sAi = 1; d.sAk1 = 0; d.sAk2 = np; d.sBk1 = 0; d.sBk2 = np; d.sBj = 1; d.sCi = np; d.sCj = 1; d.conjA = 1;
+        d.sAi = 1; d.sAk1 = 0; d.sAk2 = np; d.sBk1 = 0; d.sBk2 = np; d.sBj = 1; d.sCi = np; d.sCj = 1; d.conjA = 1; d.upper = 0; d.herm = 1;
         flops += 8.0 * ((double)nb * np * np + (double)nb * nb * np + (double)np * np * nb);
     }
     if ((rc = scratch_reserve(ctx, ctx->s_lapw_tab, 3 * (size_t)nk * sizeof(ZGemmBatch)))) return rc;

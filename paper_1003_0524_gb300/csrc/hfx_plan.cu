@@ -19,6 +19,7 @@
 // apply needs (one v_t(q) per column range).  The q sum of Eq. (vec-mat-vec)
 // is accumulated per k in FP64 in batch order, ascending q inside a batch.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -57,6 +58,44 @@ Geometry boxes(hfx_ctx *ctx) {
         g.ddim[x] = (g.tlo[x] + g.tdim[x] - 1 - pmin[x]) - g.dlo[x] + 1;
     }
     return g;
+}
+
+// The points K = G + G1 - G0 of the T box that some pair can need (G in any aux list,
+// G1 in any plane-wave list, -G0 in {0, 1}^3), ascending.
+std::vector<int> reachable(hfx_ctx *ctx, const Geometry &g) {
+    const long long box = (long long)g.tdim[0] * g.tdim[1] * g.tdim[2];
+    auto distinct = [](const std::vector<const std::vector<int> *> &lists) {
+        std::vector<std::array<int, 3>> out;
+        for (auto *l : lists)
+            for (size_t i = 0; i + 2 < l->size(); i += 3) out.push_back({(*l)[i], (*l)[i + 1], (*l)[i + 2]});
+        std::sort(out.begin(), out.end());
+        out.erase(std::unique(out.begin(), out.end()), out.end());
+        return out;
+    };
+    std::vector<const std::vector<int> *> la, lp;
+    for (auto &q : ctx->qp) la.push_back(&q.G);
+    for (auto &k : ctx->kp) lp.push_back(&k.G);
+    const auto ga = distinct(la), gp = distinct(lp);
+    // (a sum set too large to enumerate on the host: every point)
+    const bool all = (double)ga.size() * (double)gp.size() > 2e8;
+    std::vector<char> on((size_t)box, all ? 1 : 0);
+    for (size_t i = 0; i < ga.size() && !all; ++i)
+        for (auto &b : gp) {
+            const auto &a = ga[i];
+            on[((size_t)(a[0] + b[0] - g.tlo[0]) * g.tdim[1] + (a[1] + b[1] - g.tlo[1])) * g.tdim[2] + (a[2] + b[2] - g.tlo[2])] = 1;
+        }
+    // -G0: every set point also reaches its neighbours at +1 (descending: each shift once)
+    for (int x = 0; x < 3; ++x) {
+        const long long step = x == 0 ? (long long)g.tdim[1] * g.tdim[2] : (x == 1 ? g.tdim[2] : 1);
+        for (long long i = box - 1; i >= step; --i) {
+            const int c = (int)(x == 0 ? i / step : (x == 1 ? (i / step) % g.tdim[1] : i % g.tdim[2]));
+            if (c > 0 && on[i - step]) on[i] = 1;
+        }
+    }
+    std::vector<int> list;
+    for (long long i = 0; i < box; ++i)
+        if (on[i]) list.push_back((int)i);
+    return list;
 }
 
 // band block of the Z^H Y tiles: a multiple of 8 up to 64.  A tile's MMA work
@@ -130,9 +169,12 @@ struct BuildPlan {
     long long tbox = 0, dbox = 0, RSc = 0;
     int N0 = 0, sparse = 0, nb_max = 0, no_max = 0, npw_max = 0, maxD = 0, N0pad = 0, Dpad = 0, HS = 0, RS = 0, MP = 0;
     int NB = 8;
+    int ksplit = 1;                   // FP64 build: parts the sum over m of one pair is split into
     size_t o_A = 0, o_c = 0, o_G = 0, o_Ga = 0, o_npw = 0, o_nb = 0, o_no = 0, o_B = 0, o_T = 0, o_vacc = 0, o_V = 0;
     bool kp = false;                  // the k.p term at q = 0 is added
     bool inv = false;                 // inversion symmetry: packed real bands (Sec. III.D)
+    size_t o_reach = 0;               // T box points that are needed (FP64 build)
+    int nreach = 0;
     size_t o_sym = 0;                 // row operations Z' = S^H Z
     int nsym = 0;
     size_t o_eps = 0, o_p = 0, o_kp = 0;
@@ -239,6 +281,14 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
     const long long RSc = pl.RSc;
     pl.NB = gemm2_check_nb(ctx->opt.tile_nb_zhy) ? ctx->opt.tile_nb_zhy : pick_nb_zhy(pl.nb_max);
     const int NB = pl.NB;
+    if (!tc) {
+        // Z^H Y has one output per band pair: split its sum over the occupied bands
+        // until the blocks fill the SMs several times over (8 per SM evens out a wave)
+        const int T = zgemm64_tile(pl.nb_max, pl.nb_max, 1LL << 20), nt = (pl.nb_max + T - 1) / T;
+        const long long blocks = (long long)kset.size() * nk * nt * nt;
+        pl.ksplit = (int)std::max<long long>(1, std::min<long long>({(152LL * 8 + blocks - 1) / blocks, (long long)pl.no_max, 16LL}));
+    }
+    const int ksplit = pl.ksplit;
 
     // hno: occupied bands (the q->0 and k.p terms); hnom: occupied columns of k' in
     // the projections (with inversion symmetry two real bands share a column)
@@ -310,6 +360,11 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         pl.o_sym = tab.put(ops);
     }
 
+    if (!tc) {
+        const std::vector<int> list = reachable(ctx, pl.geo);
+        pl.nreach = (int)list.size();
+        pl.o_reach = tab.put(list);
+    }
     // ---- per-build products on the tensor cores (plans; their scratch is reserved below)
     if (tc) {
         if ((rc = thetapsi_tc_plan(ctx, kset, pl.geo.ddim, pl.geo.tdim, toff, tab, pl.tp))) return rc;
@@ -332,7 +387,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
     auto pair_bytes = [&](int ik, int ikp) {
         const long long nc = (long long)hnom[ikp] * hnb[ik];
         size_t praw = tc ? (size_t)((hnb[ik] + NB - 1) / NB) * ((hnb[ik] + NB - 1) / NB) * (2 * NB) * (2 * NB) * sizeof(double)
-                         : (size_t)hnb[ik] * hnb[ik] * sizeof(double2);
+                         : (size_t)ksplit * hnb[ik] * hnb[ik] * sizeof(double2);
         size_t b = (size_t)nc * RSc * sizeof(V) + praw + (size_t)nc * RSc * sizeof(double2);
         if (tc) b += (size_t)2 * 4 * nc * pl.RS * sizeof(__nv_bfloat16) + 2 * nc * sizeof(int);
         return b;
@@ -415,10 +470,10 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
             pl.flops += f * m * n * (nnz + (double)qd.naux * n) + f * m * n * ctx->nlmp * nmt +
                         f * m * n * qd.nipw * hnpw[pr.ikp];
             pl.fl_apply += f * m * n * (double)qd.D * qd.D;
-            // as executed: the upper triangle (sliced path), over the packed columns
+            // as executed: the upper triangle, over the packed columns
             // (two real parts of Y' per column with a real v_t)
             const double mc = pr.no, fe = pl.inv ? 4.0 : 8.0;
-            pl.fl_apply_exec += tc ? fe * mc * n * 0.5 * (double)qd.D * (qd.D + 1) : 8.0 * mc * n * (double)qd.D * qd.D;
+            pl.fl_apply_exec += (tc ? fe : 8.0) * mc * n * 0.5 * (double)qd.D * (qd.D + 1);
             pl.fl_zhy += f * m * n * (double)qd.naux * n;
             pl.fl_zipw += f * m * n * (double)qd.nipw * hnpw[pr.ikp];
         }
@@ -434,7 +489,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         long long praw = 0;
         for (auto &pr : bt.pairs) {
             if (tc) { long long nblk = (pr.nb + NB - 1) / NB; praw += nblk * nblk * (2 * NB) * (2 * NB); }
-            else praw += 2LL * pr.nb * pr.nb;
+            else praw += 2LL * ksplit * pr.nb * pr.nb;
         }
         bt.praw_tot = praw;
         max_praw = std::max(max_praw, praw);
@@ -476,7 +531,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         for (int i = 0; i < npairs; ++i) {
             praw_off[i] = po;
             if (tc) { long long nblk = (bt.pairs[i].nb + NB - 1) / NB; po += nblk * nblk * (2 * NB) * (2 * NB); }
-            else po += 2LL * bt.pairs[i].nb * bt.pairs[i].nb;
+            else po += 2LL * ksplit * bt.pairs[i].nb * bt.pairs[i].nb;
         }
         // per-k pair lists (ascending q) for the reduction
         std::vector<int> klist, kstart, klpairs;
@@ -517,41 +572,50 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
             bt.o_g1t = tab.put(t1);
             bt.o_g2t = tab.put(t2);
         } else {
-            std::vector<ZGemmBatch> g1(nq), g2(npairs);
+            std::vector<ZGemmBatch> g1(nq), g2((size_t)npairs * ksplit);
             for (int i = 0; i < nq; ++i) {
+                // the dense-block rows of U: columns [N0, naux) of the rows of v_t
                 const QDesc &q = bt.qd[i];
                 ZGemmBatch &b = g1[i];
-                b.A = ctx->qp[q.iq].d_VD;
-                b.B = reinterpret_cast<const double2 *>(Zc) + q.colbase * RSc;
+                b.A = ctx->qp[q.iq].d_VD + N0;
+                b.B = reinterpret_cast<const double2 *>(Zc) + q.colbase * RSc + N0;
                 b.C = Y + q.colbase * RSc + N0;
                 b.M = q.D;
                 b.N = (int)q.ncols;
                 b.K1 = 1;
-                b.K2 = q.naux;
+                b.K2 = q.D;
                 b.sAi = q.naux; b.sAk2 = 1; b.sAk1 = 0;
                 b.sBk2 = 1; b.sBk1 = 0; b.sBj = RSc;
                 b.sCi = 1; b.sCj = RSc;
                 b.conjA = 0;
+                b.upper = 1;
+                b.herm = 0;
                 bt.maxM1 = std::max(bt.maxM1, b.M);
                 bt.maxN1 = std::max(bt.maxN1, b.N);
             }
             for (int i = 0; i < npairs; ++i) {
                 const PairDesc &pr = bt.pairs[i];
                 const QDesc &q = bt.qd[pr.qslot];
-                ZGemmBatch &b = g2[i];
-                b.A = reinterpret_cast<const double2 *>(Zc) + pr.col0 * RSc;
-                b.B = Y + pr.col0 * RSc;
-                b.C = reinterpret_cast<double2 *>(praw + praw_off[i]);
-                b.M = pr.nb;
-                b.N = pr.nb;
-                b.K1 = pr.no;
-                b.K2 = q.naux;
-                b.sAi = RSc; b.sAk1 = (long long)pr.nb * RSc; b.sAk2 = 1;
-                b.sBk1 = (long long)pr.nb * RSc; b.sBk2 = 1; b.sBj = RSc;
-                b.sCi = pr.nb; b.sCj = 1;
-                b.conjA = 1;
                 bt.mx2 = std::max(bt.mx2, pr.nb);
-                if (pr.no == 0) { b.K1 = 1; b.K2 = 0; }
+                for (int s2 = 0; s2 < ksplit; ++s2) {
+                    // occupied bands [m0, m1) of the pair (empty parts write zeros)
+                    const int m0 = (int)((long long)pr.no * s2 / ksplit), m1 = (int)((long long)pr.no * (s2 + 1) / ksplit);
+                    ZGemmBatch &b = g2[(size_t)i * ksplit + s2];
+                    b.A = reinterpret_cast<const double2 *>(Zc) + (pr.col0 + (long long)m0 * pr.nb) * RSc;
+                    b.B = Y + (pr.col0 + (long long)m0 * pr.nb) * RSc;
+                    b.C = reinterpret_cast<double2 *>(praw + praw_off[i]) + (size_t)s2 * pr.nb * pr.nb;
+                    b.M = pr.nb;
+                    b.N = pr.nb;
+                    b.K1 = m1 - m0;
+                    b.K2 = q.naux;
+                    b.sAi = RSc; b.sAk1 = (long long)pr.nb * RSc; b.sAk2 = 1;
+                    b.sBk1 = (long long)pr.nb * RSc; b.sBk2 = 1; b.sBj = RSc;
+                    b.sCi = pr.nb; b.sCj = 1;
+                    b.conjA = 1;
+                    b.upper = 0;
+                    b.herm = 0;
+                    if (m1 == m0) { b.K1 = 1; b.K2 = 0; }
+                }
             }
             bt.o_zg1 = tab.put(g1);
             bt.o_zg2 = tab.put(g2);
@@ -601,7 +665,7 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             ++nl;
             if (!tc) {
                 launch_thetapsi<R>(reinterpret_cast<double2 *>(ctx->s_theta.p), pl.geo.dlo, pl.geo.ddim, pl.geo.tlo,
-                                   pl.geo.tdim, ctx->kp[ik].d_c, ctx->kp[ik].d_G, ctx->kp[ik].nb, ctx->kp[ik].npw,
+                                   pl.geo.tdim, reinterpret_cast<const int *>(tab + pl.o_reach), pl.nreach, ctx->kp[ik].d_c, ctx->kp[ik].d_G, ctx->kp[ik].nb, ctx->kp[ik].npw,
                                    at<V>(ctx->s_thpsi.p, to[ik] * sizeof(V)), ctx->stream);
                 ++nl;
             }
@@ -733,7 +797,7 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             launch_block64(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb),
                            reinterpret_cast<const double2 *>(Zc), Yd, RSc, nch, P, N0, bt.maxcols, ctx->stream);
             rec(ctx, bt.ev[8]);
-            launch_zgemm64(reinterpret_cast<const ZGemmBatch *>(tab + bt.o_zg2), npairs, bt.mx2, bt.mx2, ctx->stream);
+            launch_zgemm64(reinterpret_cast<const ZGemmBatch *>(tab + bt.o_zg2), npairs * pl.ksplit, bt.mx2, bt.mx2, ctx->stream);
             rec(ctx, bt.ev[9]);
             nl += 3;
             if ((rc = cuda_check(ctx, cudaGetLastError(), "fp64 contraction"))) return rc;
@@ -741,7 +805,7 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
         launch_reduce_pairs(d_pairs, reinterpret_cast<const int *>(tab + bt.o_kstart),
                             reinterpret_cast<const int *>(tab + bt.o_klp), bt.nklist,
                             reinterpret_cast<const int *>(tab + bt.o_klist), praw, d_praw_off, pl.NB,
-                            tc ? ((pl.inv && gemm2_real_form(pl.NB)) ? 2 : 1) : 0,
+                            tc ? ((pl.inv && gemm2_real_form(pl.NB)) ? 2 : 1) : 0, pl.ksplit,
                             pl.inv ? 1 : 0, reinterpret_cast<double2 *const *>(tab + pl.o_vacc),
                             reinterpret_cast<const int *>(tab + pl.o_nb),
                             pl.nb_max, ctx->stream);
