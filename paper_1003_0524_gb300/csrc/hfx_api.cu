@@ -400,44 +400,41 @@ int hfx_set_coulomb(hfx_ctx *ctx, int iq, int n_ipw, const int *G_aux, const dou
     const int naux = ctx->nmt + n_ipw;
     if (ld < naux) return set_err(ctx, HFX_EINVAL, "set_coulomb: leading dimension below N_aux");
     const size_t nv = (size_t)naux * naux;
-    // rows of stride ld into one contiguous N_aux x N_aux copy
-    std::vector<double> vc;
-    const double *vv = v;
-    if (ld != naux) {
-        vc.resize(2 * nv);
-        for (int i = 0; i < naux; ++i) std::memcpy(vc.data() + 2 * (size_t)i * naux, v + 2 * (size_t)i * ld, 16 * (size_t)naux);
-        vv = vc.data();
-    }
-    if (!finite_all(vv, 2 * nv)) return set_err(ctx, HFX_ENONFINITE, "set_coulomb: non-finite element");
-    double mx = 0.0, dev = 0.0;
-    for (size_t i = 0; i < 2 * nv; ++i) mx = std::max(mx, std::fabs(vv[i]));
-    for (int i = 0; i < naux; ++i)
-        for (int j = 0; j <= i; ++j) {
-            const double *a = vv + 2 * ((size_t)i * naux + j), *b = vv + 2 * ((size_t)j * naux + i);
-            dev = std::max(dev, std::fabs(a[0] - b[0]) + std::fabs(a[1] + b[1]));
-        }
-    if (dev > ctx->opt.herm_tol * std::max(mx, 1e-300)) return set_err(ctx, HFX_ENOTHERM, "set_coulomb: v(q) is not Hermitian");
-    std::vector<double> vreal;
-    if (ctx->opt.inversion) {
-        // over the symmetrized MT functions of Sec. III.D, v(q) is real
-        double im = 0.0;
-        for (size_t i = 0; i < nv; ++i) im = std::max(im, std::fabs(vv[2 * i + 1]));
-        if (im > ctx->opt.herm_tol * std::max(mx, 1e-300))
-            return set_err(ctx, HFX_EINVAL, "set_coulomb: v(q) over the symmetrized basis is not real (inversion mode)");
-        vreal.assign(vv, vv + 2 * nv);
-        for (size_t i = 0; i < nv; ++i) vreal[2 * i + 1] = 0.0;
-        vv = vreal.data();
-    }
+    // v goes to a staging buffer of the context, is checked there on the device (three
+    // host passes over the matrix took four fifths of this call) and copied to its
+    // place only when it passes: a refused v leaves the one before it as it was
+    int rc = cuda_check(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
+    if (rc) return rc;
+    if ((rc = scratch_reserve(ctx, ctx->s_qd, nv * sizeof(double2) + sizeof(CoulombCheck)))) return rc;
+    double2 *d_in = reinterpret_cast<double2 *>(ctx->s_qd.p);
+    CoulombCheck *d_chk = reinterpret_cast<CoulombCheck *>(d_in + nv), chk;
+    if ((rc = cuda_check(ctx, cudaMemcpy2DAsync(d_in, 16 * (size_t)naux, v, 16 * (size_t)ld, 16 * (size_t)naux, naux,
+                                                cudaMemcpyHostToDevice, ctx->stream), "copy to device")))
+        return rc;
+    launch_check_coulomb(d_in, naux, ctx->opt.inversion ? 1 : 0, d_chk, ctx->stream);
+    if ((rc = cuda_check(ctx, cudaGetLastError(), "set_coulomb check")) ||
+        (rc = cuda_check(ctx, cudaMemcpyAsync(&chk, d_chk, sizeof(chk), cudaMemcpyDeviceToHost, ctx->stream), "set_coulomb check")) ||
+        (rc = sync(ctx)))
+        return rc;
+    if (chk.nonfinite) return set_err(ctx, HFX_ENONFINITE, "set_coulomb: non-finite element");
+    double mx, dev, im;
+    std::memcpy(&mx, &chk.mx, 8);
+    std::memcpy(&dev, &chk.dev, 8);
+    std::memcpy(&im, &chk.im, 8);
+    const double tol = ctx->opt.herm_tol * std::max(mx, 1e-300);
+    if (dev > tol) return set_err(ctx, HFX_ENOTHERM, "set_coulomb: v(q) is not Hermitian");
+    // over the symmetrized MT functions of Sec. III.D, v(q) is real
+    if (ctx->opt.inversion && im > tol)
+        return set_err(ctx, HFX_EINVAL, "set_coulomb: v(q) over the symmetrized basis is not real (inversion mode)");
     QPoint &q = ctx->qp[iq];
     if (q.set && q.nipw != n_ipw) {
         dfree(q.d_G); dfree(q.d_v); dfree(q.d_VD); dfree(q.d_VB);
         q.d_G = nullptr; q.d_v = nullptr; q.d_VD = nullptr; q.d_VB = nullptr;
         q.vd_cap = q.vb_cap = 0;
     }
-    int rc = HFX_OK;
     if (!q.d_v && ((rc = dalloc(ctx, &q.d_G, (size_t)3 * std::max(n_ipw, 1))) || (rc = dalloc(ctx, &q.d_v, nv))))
         return rc;
-    if ((rc = h2d(ctx, q.d_G, G_aux, (size_t)3 * n_ipw)) || (rc = h2d(ctx, q.d_v, reinterpret_cast<const double2 *>(vv), nv)) ||
+    if ((rc = h2d(ctx, q.d_G, G_aux, (size_t)3 * n_ipw)) || (rc = cuda_check(ctx, cudaMemcpyAsync(q.d_v, d_in, nv * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "copy v")) ||
         (rc = sync(ctx)))
         return rc;
     if (!q.set || q.nipw != n_ipw || q.G.size() != (size_t)3 * n_ipw ||

@@ -243,6 +243,12 @@ void launch_transform_v(const double2 *d_v, double2 *d_VD, double2 *d_VB, const 
 // row of U adjacent (complex path), else in two blocks (real path).
 void launch_build_ap(const double2 *d_VD, __nv_bfloat16 *d_Ap, int *d_aexp, int D, int naux, int N0, int N0pad,
                      int Dpad, int RS, int interleave, cudaStream_t st);
+// What set_coulomb checks of v: a non-finite element, max |component|, max
+// |v_ij - conj(v_ji)| (1-norm of the components) and max |Im|, as bit patterns
+// (non-negative doubles order like theirs).  zero_im: v is real up to tolerance and
+// its imaginary parts are set to zero after the check.
+struct CoulombCheck { unsigned long long mx, dev, im; int nonfinite, pad; };
+void launch_check_coulomb(double2 *d_v, int naux, int zero_im, CoulombCheck *d_chk, cudaStream_t st);
 // q->0 bracket of Eq. (div final) into *d_out (FP64); d_partial holds
 // q0_partial_count() doubles.
 void launch_q0_bracket_impl(double *d_out, double *d_partial, const int mesh[3], const double *B, double omega,

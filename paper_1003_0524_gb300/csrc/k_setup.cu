@@ -316,6 +316,64 @@ __global__ void build_ap_kernel(const double2 *VD, __nv_bfloat16 *Ap, int *aexp,
     }
 }
 
+// The checks of set_coulomb: one block per pair of 32 x 32 tiles (I, J), J <= I, both
+// read along their rows and compared through shared memory.  Bound by memory (16 bytes
+// per element, read once); comparisons of magnitudes run on the integer units.
+__global__ void __launch_bounds__(256) check_coulomb_kernel(double2 *__restrict__ v, int n, int zero_im,
+                                                            CoulombCheck *__restrict__ chk) {
+    int I = 0, J = blockIdx.x;   // row of the triangle of tile pairs
+    {
+        I = (int)((sqrtf(8.0f * (float)J + 1.0f) - 1.0f) * 0.5f);
+        while ((long long)(I + 1) * (I + 2) / 2 <= J) ++I;
+        while ((long long)I * (I + 1) / 2 > J) --I;
+        J -= (int)((long long)I * (I + 1) / 2);
+    }
+    __shared__ double2 b[32][33];
+    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+    unsigned long long mx = 0, dev = 0, im = 0;
+    bool bad = false;
+    auto look = [&](const double2 &x) {
+        const unsigned long long r = tc::abs_bits(x.x), i = tc::abs_bits(x.y);
+        bad |= r >= 0x7ff0000000000000ULL || i >= 0x7ff0000000000000ULL;
+        mx = max(mx, max(r, i));
+        im = max(im, i);
+    };
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int i = J * 32 + ty + 8 * s, j = I * 32 + tx;   // tile (J, I)
+        double2 x = make_double2(0.0, 0.0);
+        if (i < n && j < n) {
+            x = v[(size_t)i * n + j];
+            look(x);
+            if (zero_im && I != J) v[(size_t)i * n + j].y = 0.0;
+        }
+        b[ty + 8 * s][tx] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int i = I * 32 + ty + 8 * s, j = J * 32 + tx;   // tile (I, J)
+        if (i >= n || j >= n) continue;
+        const double2 x = I == J ? b[ty + 8 * s][tx] : v[(size_t)i * n + j], y = b[tx][ty + 8 * s];
+        look(x);
+        dev = max(dev, tc::abs_bits(fabs(x.x - y.x) + fabs(x.y + y.y)));
+        if (zero_im) v[(size_t)i * n + j].y = 0.0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        dev = max(dev, __shfl_xor_sync(0xffffffffu, dev, o));
+        im = max(im, __shfl_xor_sync(0xffffffffu, im, o));
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if (tx == 0) {
+        atomicMax(&chk->mx, mx);
+        atomicMax(&chk->dev, dev);
+        atomicMax(&chk->im, im);
+        if (bad) chk->nonfinite = 1;
+    }
+}
+
 // Partial sums of e^{-beta|x|^2}/|x|^2 over the vectors x = q + G, 0 < |x| <= q0,
 // of every q of the mesh.  Together they are the lattice of the b_i / m_i, so the
 // sum runs over its lines (X, Y) along b_2 / m_2, over the half of them that
@@ -479,6 +537,12 @@ void launch_transform_v(const double2 *d_v, double2 *d_VD, double2 *d_VB, const 
 void launch_build_ap(const double2 *d_VD, __nv_bfloat16 *d_Ap, int *d_aexp, int D, int naux, int N0, int N0pad,
                      int Dpad, int RS, int interleave, cudaStream_t st) {
     build_ap_kernel<<<2 * Dpad, 256, 0, st>>>(d_VD, d_Ap, d_aexp, D, naux, N0, N0pad, Dpad, RS, interleave);
+}
+
+void launch_check_coulomb(double2 *d_v, int naux, int zero_im, CoulombCheck *d_chk, cudaStream_t st) {
+    cudaMemsetAsync(d_chk, 0, sizeof(CoulombCheck), st);
+    const long long nt = (naux + 31) / 32, blocks = nt * (nt + 1) / 2;
+    check_coulomb_kernel<<<(unsigned)blocks, 256, 0, st>>>(d_v, naux, zero_im, d_chk);
 }
 
 // q->0 bracket.
