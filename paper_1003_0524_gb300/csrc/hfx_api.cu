@@ -630,7 +630,7 @@ int prepare_coulomb(hfx_ctx *ctx) {
         int maxD = 0;
         for (auto &q : ctx->qp) maxD = std::max(maxD, ctx->nmt + q.nipw - ctx->N0);
         int N0pad = (int)rup(ctx->N0, 64), Dpad = (int)rup(maxD, 128);
-        int RS = 2 * (N0pad + Dpad), MP = 2 * Dpad;
+        int HS = slice_half(N0pad, maxD), RS = 2 * HS, MP = 2 * Dpad;
         size_t per = (size_t)4 * MP * RS;
         if ((rc = scratch_reserve(ctx, ctx->s_ap, per * ctx->nk * sizeof(__nv_bfloat16))) ||
             (rc = scratch_reserve(ctx, ctx->s_aexp, (size_t)MP * ctx->nk * sizeof(int))))
@@ -642,7 +642,7 @@ int prepare_coulomb(hfx_ctx *ctx) {
             int naux = ctx->nmt + q.nipw;
             // the complex path interleaves the real and imaginary rows of U; the real
             // path (inversion symmetry) keeps them in two blocks
-            launch_build_ap(q.d_VD, ap + per * iq, aexp + (size_t)MP * iq, naux - ctx->N0, naux, ctx->N0, N0pad, Dpad, RS,
+            launch_build_ap(q.d_VD, ap + per * iq, aexp + (size_t)MP * iq, naux - ctx->N0, naux, ctx->N0, N0pad, HS, MP, RS,
                             ctx->opt.inversion ? 0 : 1, ctx->stream);
         }
         if ((rc = cuda_check(ctx, cudaGetLastError(), "slice embedding")) || (rc = sync(ctx))) return rc;

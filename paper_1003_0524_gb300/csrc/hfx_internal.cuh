@@ -242,7 +242,7 @@ void launch_transform_v(const double2 *d_v, double2 *d_VD, double2 *d_VB, const 
 // of v_t with half its diagonal; interleave: the real and imaginary rows of each
 // row of U adjacent (complex path), else in two blocks (real path).
 void launch_build_ap(const double2 *d_VD, __nv_bfloat16 *d_Ap, int *d_aexp, int D, int naux, int N0, int N0pad,
-                     int Dpad, int RS, int interleave, cudaStream_t st);
+                     int HS, int MP, int RS, int interleave, cudaStream_t st);
 // What set_coulomb checks of v: a non-finite element, max |component|, max
 // |v_ij - conj(v_ji)| (1-norm of the components) and max |Im|, as bit patterns
 // (non-negative doubles order like theirs).  zero_im: v is real up to tolerance and
@@ -308,7 +308,11 @@ void launch_block64(const QDesc *d_q, int nq, const double2 *const *d_VB, const 
 // ------------------------------------------------------------ kernels (tensor-core contraction, k_contract_tc.cu)
 template <typename V>
 void launch_slice_cols(const V *d_Z, long long RSc, const QDesc *d_q, int nq, long long NC, long long maxcols, int N0,
-                       int N0pad, int Dpad, int RS, __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st);
+                       int N0pad, int HS, int RS, __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st);
+// The slices of Z with the interstitial rows still in the G-major plane ZI [g][NCi].
+int launch_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long NCi, const double2 *d_Z, long long RSc, const QDesc *d_q,
+                   int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
+                   __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st);
 // The channel blocks of Y' = U Z (rows [0, N0)), U the upper triangle of v_t
 // with half its diagonal.  (With d_VD non-null, the double-FP32 kernel would
 // also add the dense rows' couplings to the mu = 0 functions, the lower
@@ -317,6 +321,10 @@ template <typename V>
 void launch_block_y(const QDesc *d_q, int nq, const double2 *const *d_VB, const double2 *const *d_VD, const V *d_Z,
                     double2 *d_Y, long long RSc, int P, int N0, long long maxcols, cudaStream_t st);
 bool block_y_couples(int P, int N0);
+// Half width of the slice rows: the mu = 0 rows (N0pad) and the dense rows, padded to a
+// multiple of 128.  (64 would save 8 % of the planes of the 2-atom workload, but its
+// rows of 22 x 128 bytes cost the Coulomb apply 7 %: 13.2 against 12.3 ms.)
+inline int slice_half(int N0pad, int maxD) { return N0pad + (maxD + 127) / 128 * 128; }
 // GEMM1 tiles of one batch (host) and its launch: Y' = U Z for the dense-block
 // rows, U the upper triangle of v_t with half its diagonal (the slices of
 // launch_build_ap), K of every row tile from its first row on.
@@ -325,7 +333,7 @@ bool block_y_couples(int P, int N0);
 int gemm1_tiles(const QDesc *h_q, int nq, int N0pad, bool real_v, std::vector<unsigned char> &out);
 int launch_gemm1_tc(hfx_ctx *ctx, const __nv_bfloat16 *d_Ap_all, long long ap_rows, const int *d_aexp, const QDesc *d_q,
                     const __nv_bfloat16 *d_ZS, const int *d_zexp, double2 *d_Y, long long RSc, long long NC, int N0,
-                    int N0pad, int Dpad, int RS, const void *d_tiles, int ntiles);
+                    int N0pad, int HS, int MP, int RS, const void *d_tiles, int ntiles);
 // real_form: the Z^H Y tiles of the inversion-symmetric path (only Re P', two
 // row blocks per tile; band blocks of 16, 32, 48 or 64, see gemm2_real_form)
 int gemm2_tiles(const PairDesc *h_pairs, int npairs, int NB, bool real_form, std::vector<unsigned char> &out);
@@ -362,12 +370,12 @@ int zipw_tc_plan_batch(hfx_ctx *ctx, const ZipwBuild &zb, const std::vector<int>
                        HostArena &tab, ZipwBatch &bt);
 int zipw_tc_run_build(hfx_ctx *ctx, const ZipwBuild &zb, const char *dtab, char *dscr, const double2 *const *d_ck,
                       const int *const *d_Gk, const int *d_npw, const double2 *const *d_Tk, const int *d_nb);
-// The interstitial rows come out G-major into d_ZI [g][NCi] (the kernel's
-// stores then fill whole sectors) and are transposed into d_Z after the kernel.
+// The interstitial rows come out G-major into d_ZI [g][NCi] (the kernel's stores then
+// fill whole sectors); with transpose they are also put into d_Z after the kernel.
 int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, const char *dtab, const char *dscr,
                       __nv_bfloat16 *dTq, const PairDesc *d_pairs, const double2 *const *d_Tk, const int *d_nb,
                       double2 *d_Z, long long RSc, double2 *d_ZI, long long NCi, const QDesc *d_qd, int nq,
-                      long long maxcols, int max_nipw, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch);
+                      long long maxcols, int max_nipw, bool transpose, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch);
 
 // ------------------------------------------------------------ stage-1 products on the tensor cores (k_cgemm_tc.cu)
 struct TpPlan {                             // T_n(K) of every k of the build (Sec. III.B)

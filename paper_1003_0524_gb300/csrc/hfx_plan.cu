@@ -275,7 +275,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
     pl.RSc = naux_max;
     pl.N0pad = (int)rup(N0, 64);
     pl.Dpad = (int)rup(pl.maxD, 128);
-    pl.HS = pl.N0pad + pl.Dpad;
+    pl.HS = slice_half(pl.N0pad, pl.maxD);
     pl.RS = 2 * pl.HS;
     pl.MP = 2 * pl.Dpad;
     const long long RSc = pl.RSc;
@@ -708,16 +708,19 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             ++nl;
         }
         rec(ctx, bt.ev[1]);
+        // the slicing kernel reads the interstitial rows where the interstitial kernel
+        // left them; only a caller's projections or keep_products need them in Z
+        const bool z_whole = keep || !bt.overrides.empty();
+        int max_nipw = 0;
+        for (auto &q : bt.qd) max_nipw = std::max(max_nipw, q.nipw);
         if (tc && sizeof(R) == 8) {
             // the G-major output plane of the interstitial kernel lives in the Y buffer,
             // which is free until the Coulomb apply
-            int max_nipw = 0;
-            for (auto &q : bt.qd) max_nipw = std::max(max_nipw, q.nipw);
             if ((rc = zipw_tc_run_batch(ctx, pl.zipw, bt.zipw, tab, reinterpret_cast<char *>(ctx->s_zipw.p),
                                         at<__nv_bfloat16>(ctx->s_zipw.p, pl.zipw_tq_off), d_pairs,
                                         reinterpret_cast<const double2 *const *>(tab + pl.o_T),
                                         reinterpret_cast<const int *>(tab + pl.o_nb), reinterpret_cast<double2 *>(Zc), RSc,
-                                        reinterpret_cast<double2 *>(ctx->s_y64.p), bt.ncols, d_qd, nq, bt.maxcols, max_nipw,
+                                        reinterpret_cast<double2 *>(ctx->s_y64.p), bt.ncols, d_qd, nq, bt.maxcols, max_nipw, z_whole,
                                         bt.ev[2], bt.ev[3], &nl)))
                 return rc;
         } else {
@@ -766,20 +769,25 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             __nv_bfloat16 *ZS = reinterpret_cast<__nv_bfloat16 *>(ctx->s_zs.p), *YS = reinterpret_cast<__nv_bfloat16 *>(ctx->s_ys.p);
             double2 *Yd = reinterpret_cast<double2 *>(ctx->s_y64.p);
             int *zexp = reinterpret_cast<int *>(ctx->s_xexp.p), *yexp = zexp + bt.ncols;
-            launch_slice_cols<V>(Zc, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.Dpad, pl.RS, ZS, zexp, ctx->stream);
-            if ((rc = cuda_check(ctx, cudaGetLastError(), "slice kernels"))) return rc;
+            if (z_whole || !bt.zipw.ok) {
+                launch_slice_cols<V>(Zc, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.HS, pl.RS, ZS, zexp, ctx->stream);
+                if ((rc = cuda_check(ctx, cudaGetLastError(), "slice kernels"))) return rc;
+            } else if ((rc = launch_slice_z(ctx, Yd, bt.ncols, reinterpret_cast<double2 *>(Zc), RSc, d_qd, nq, bt.ncols,
+                                            bt.maxcols, nmt, N0, pl.N0pad, pl.HS, pl.RS, ZS, zexp, ctx->stream))) {
+                return rc;
+            }
             rec(ctx, bt.ev[6]);
             // Y' = U Z with U the upper triangle of v_t (half diagonal): the dense
             // rows on the tensor cores, the mu = 0 rows in the channel-block kernel;
             // the q reduction adds P' + P'^H for P' = Z^H Y'
             if ((rc = launch_gemm1_tc(ctx, reinterpret_cast<const __nv_bfloat16 *>(ctx->s_ap.p), (long long)nk * 4 * pl.MP,
                                       reinterpret_cast<const int *>(ctx->s_aexp.p), d_qd, ZS, zexp, Yd, RSc, bt.ncols, N0,
-                                      pl.N0pad, pl.Dpad, pl.RS, tab + bt.o_g1t, bt.n_g1t)))
+                                      pl.N0pad, pl.HS, pl.MP, pl.RS, tab + bt.o_g1t, bt.n_g1t)))
                 return rc;
             rec(ctx, bt.ev[7]);
             launch_block_y<V>(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb), nullptr, Zc, Yd, RSc, P,
                               N0, bt.maxcols, ctx->stream);
-            launch_slice_cols<double2>(Yd, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.Dpad, pl.RS, YS, yexp,
+            launch_slice_cols<double2>(Yd, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.HS, pl.RS, YS, yexp,
                                        ctx->stream);
             rec(ctx, bt.ev[8]);
             if ((rc = launch_gemm2_tc(ctx, ZS, YS, zexp, yexp, bt.ncols, pl.RS, pl.HS, pl.N0pad, d_pairs, d_qd, pl.NB,

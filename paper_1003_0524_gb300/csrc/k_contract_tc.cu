@@ -43,19 +43,14 @@ namespace {
 // For every column of the batch: exponent over its rows (real and imaginary
 // parts of rows [0, N0) and [N0, N0 + D_q) of Zc), then slices into
 // XS[p][col][u]: u in [0, HS) real parts, [HS, 2 HS) imaginary parts (mu=0
-// rows padded to N0pad, dense rows padded to Dpad).  One warp per column; in
+// rows padded to N0pad, dense rows to HS - N0pad).  One warp per column; in
 // the slicing pass each lane takes four consecutive rows, so every plane is
 // written with 8-byte stores (N0pad and HS are multiples of 64).
-__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
 template <typename V>
 __global__ void __launch_bounds__(256, 4) slice_cols_kernel(const V *__restrict__ Z, long long RSc, const QDesc *__restrict__ qd, int N0,
-                                  int N0pad, int Dpad, int RS, long long NC, __nv_bfloat16 *__restrict__ XS,
+                                  int N0pad, int HS, int RS, long long NC, __nv_bfloat16 *__restrict__ XS,
                                   int *__restrict__ xexp) {
     const QDesc q = qd[blockIdx.y];
-    const int HS = N0pad + Dpad;
     const int wpb = blockDim.x / 32, lane = threadIdx.x % 32;
     const long long plane = NC * RS;
     for (long long c = (long long)blockIdx.x * wpb + threadIdx.x / 32; c < q.ncols; c += (long long)gridDim.x * wpb) {
@@ -77,7 +72,7 @@ __global__ void __launch_bounds__(256, 4) slice_cols_kernel(const V *__restrict_
             int row0, nvalid;
             if (u0 < N0pad) { row0 = u0; nvalid = N0 - u0; }
             else { row0 = N0 + (u0 - N0pad); nvalid = q.D - (u0 - N0pad); }
-            __nv_bfloat16 sr[4][NPL], si[4][NPL];
+            Digits sr[4], si[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 double xr = 0.0, xi = 0.0;
@@ -86,16 +81,104 @@ __global__ void __launch_bounds__(256, 4) slice_cols_kernel(const V *__restrict_
                     xr = (double)v.x;
                     xi = (double)v.y;
                 }
-                slice4(xr, e, sr[t]);
-                slice4(xi, e, si[t]);
+                sr[t] = slice4f(xr, e);
+                si[t] = slice4f(xi, e);
             }
 #pragma unroll
             for (int p = 0; p < NPL; ++p) {
-                uint2 wr = make_uint2(pack_bf16x2(sr[0][p], sr[1][p]), pack_bf16x2(sr[2][p], sr[3][p]));
-                uint2 wi = make_uint2(pack_bf16x2(si[0][p], si[1][p]), pack_bf16x2(si[2][p], si[3][p]));
+                uint2 wr = make_uint2(pack_digits(sr[0].s[p], sr[1].s[p]), pack_digits(sr[2].s[p], sr[3].s[p]));
+                uint2 wi = make_uint2(pack_digits(si[0].s[p], si[1].s[p]), pack_digits(si[2].s[p], si[3].s[p]));
                 *reinterpret_cast<uint2 *>(XS + p * plane + base + u0) = wr;
                 *reinterpret_cast<uint2 *>(XS + p * plane + base + HS + u0) = wi;
             }
+        }
+    }
+}
+
+// The same slices of the projections Z, whose interstitial rows come from the G-major
+// plane ZI [g][col] of the interstitial kernel and whose muffin-tin rows from Z: the
+// transposition, the column maximum and the slicing in one kernel.  A block takes
+// SZ_COLS = 8 adjacent columns (128 bytes of every ZI row); it reads them twice and
+// turns chunks of 128 rows around in shared memory, so that the planes are written in
+// runs of 256 bytes.  Bound by memory: two reads of Z and one write of its planes, 44
+// GB on the 2-atom workload (4x4x4 k, 40 bands) in 6.6 ms.  The transposition into Z and
+// a warp per column took 9.7 ms there.  Keeping the columns in shared memory between
+// the two reads leaves too few warps (9.4 ms), as does bounding the columns in flight
+// so that the second read hits L2 (7.6 ms); 16 columns or 128 threads change nothing.
+constexpr int SZ_COLS = 8, SZ_THREADS = 256;
+__global__ void __launch_bounds__(SZ_THREADS) slice_z_kernel(const double2 *__restrict__ ZI, long long NCi,
+                                                          const double2 *__restrict__ Z, long long RSc,
+                                                          const QDesc *__restrict__ qd, int nmt, int N0, int N0pad, int HS,
+                                                          int RS, long long NC, __nv_bfloat16 *__restrict__ XS,
+                                                          int *__restrict__ xexp) {
+    constexpr int NJ = SZ_THREADS / SZ_COLS, CH = 4 * NJ, CS = CH + 8;   // rows per pass, per chunk, padded
+    __shared__ __align__(16) __nv_bfloat16 stage[2 * NPL * SZ_COLS * CS];   // [plane][part][column][CS]
+    __shared__ unsigned long long red[SZ_THREADS / 32][SZ_COLS];
+    const QDesc q = qd[blockIdx.y];
+    const long long c0 = (long long)blockIdx.x * SZ_COLS;
+    if (c0 >= q.ncols) return;
+    const int tid = threadIdx.x, c = tid % SZ_COLS, j = tid / SZ_COLS;
+    const bool live = c0 + c < q.ncols;
+    const long long col = q.colbase + (live ? c0 + c : c0);
+    const double2 *z = Z + col * RSc, *zi = ZI + col;
+    unsigned long long mx = 0;
+    for (int i = j; i < nmt; i += NJ) {
+        const double2 v = z[i];
+        mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
+    }
+#pragma unroll 8
+    for (int g = j; g < q.nipw; g += NJ) {
+        const double2 v = zi[(size_t)g * NCi];
+        mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
+    }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+    if (tid % 32 < SZ_COLS) red[tid / 32][c] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < SZ_THREADS / 32; ++w) mx = max(mx, red[w][c]);
+    const int e = line_exp_bits(mx);
+    if (j == 0 && live) xexp[col] = e;
+    const int nd = nmt - N0;                       // muffin-tin rows among the dense ones
+    const long long plane = NC * RS;
+    double2 v[4];                                  // this thread's four rows of a chunk
+    auto fetch = [&](int u) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int dr = u + t - N0pad;          // dense row
+            v[t] = make_double2(0.0, 0.0);
+            if (dr >= nd) {
+                if (dr < q.D) v[t] = zi[(size_t)(dr - nd) * NCi];
+            } else if (dr >= 0) {
+                v[t] = z[N0 + dr];
+            } else if (u + t < N0) {
+                v[t] = z[u + t];
+            }
+        }
+    };
+    fetch(4 * j);
+    for (int u0 = 0; u0 < HS; u0 += CH) {
+        Digits sr[4], si[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            sr[t] = slice4f(v[t].x, e);
+            si[t] = slice4f(v[t].y, e);
+        }
+        if (u0 + CH < HS) fetch(u0 + CH + 4 * j);  // the next chunk, while this one is stored
+        __syncthreads();                           // the chunk before has been stored
+#pragma unroll
+        for (int p = 0; p < NPL; ++p) {
+            __nv_bfloat16 *s = stage + (size_t)((2 * p) * SZ_COLS + c) * CS + 4 * j;
+            *reinterpret_cast<uint2 *>(s) = make_uint2(pack_digits(sr[0].s[p], sr[1].s[p]), pack_digits(sr[2].s[p], sr[3].s[p]));
+            *reinterpret_cast<uint2 *>(s + SZ_COLS * CS) =
+                make_uint2(pack_digits(si[0].s[p], si[1].s[p]), pack_digits(si[2].s[p], si[3].s[p]));
+        }
+        __syncthreads();
+        for (int t = tid; t < 2 * NPL * SZ_COLS * (CH / 8); t += SZ_THREADS) {
+            const int x = t % (CH / 8), line = t / (CH / 8), cc = line % SZ_COLS, pp = line / SZ_COLS;   // pp = 2 plane + part
+            if (u0 + 8 * x >= HS || c0 + cc >= q.ncols) continue;
+            const uint4 w = *reinterpret_cast<const uint4 *>(stage + (size_t)line * CS + 8 * x);
+            __stcs(reinterpret_cast<uint4 *>(XS + (pp >> 1) * plane + (q.colbase + c0 + cc) * RS + (pp & 1) * HS + u0 + 8 * x), w);
         }
     }
 }
@@ -253,7 +336,7 @@ struct G1Params {
     double2 *Y;            // [col][RSc] (rows N0 + r)
     long long RSc;
     long long NC;          // columns of the batch (plane stride in rows of ZS)
-    int RS, HS, MP, N0pad, Dpad, N0;
+    int RS, HS, MP, N0pad, N0;
     int *err;
 };
 
@@ -788,17 +871,26 @@ int num_sms() {
 
 template <typename V>
 void launch_slice_cols(const V *d_Z, long long RSc, const QDesc *d_q, int nq, long long NC, long long maxcols, int N0,
-                       int N0pad, int Dpad, int RS, __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st) {
+                       int N0pad, int HS, int RS, __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st) {
     long long g = (maxcols + 7) / 8;
     if (g > 8192) g = 8192;
     if (g < 1) g = 1;
     dim3 grid((unsigned)g, (unsigned)nq);
-    slice_cols_kernel<V><<<grid, 256, 0, st>>>(d_Z, RSc, d_q, N0, N0pad, Dpad, RS, NC, d_XS, d_exp);
+    slice_cols_kernel<V><<<grid, 256, 0, st>>>(d_Z, RSc, d_q, N0, N0pad, HS, RS, NC, d_XS, d_exp);
 }
 template void launch_slice_cols<float2>(const float2 *, long long, const QDesc *, int, long long, long long, int, int,
                                         int, int, __nv_bfloat16 *, int *, cudaStream_t);
 template void launch_slice_cols<double2>(const double2 *, long long, const QDesc *, int, long long, long long, int, int,
                                          int, int, __nv_bfloat16 *, int *, cudaStream_t);
+
+int launch_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long NCi, const double2 *d_Z, long long RSc, const QDesc *d_q,
+                   int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
+                   __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st) {
+    if (nq == 0 || maxcols == 0) return HFX_OK;
+    const dim3 grid((unsigned)((maxcols + SZ_COLS - 1) / SZ_COLS), (unsigned)nq);
+    slice_z_kernel<<<grid, SZ_THREADS, 0, st>>>(d_ZI, NCi, d_Z, RSc, d_q, nmt, N0, N0pad, HS, RS, NC, d_XS, d_exp);
+    return cuda_check(ctx, cudaGetLastError(), "slice kernel");
+}
 
 bool block_y_couples(int P, int N0) { return P >= 2 && P <= 4 && N0 > 0 && N0 % (P - 1) == 0; }
 
@@ -868,8 +960,7 @@ int gemm1_tiles(const QDesc *h_q, int nq, int N0pad, bool real_v, std::vector<un
 
 int launch_gemm1_tc(hfx_ctx *ctx, const __nv_bfloat16 *d_Ap_all, long long ap_rows, const int *d_aexp, const QDesc *d_q,
                     const __nv_bfloat16 *d_ZS, const int *d_zexp, double2 *d_Y, long long RSc, long long NC, int N0,
-                    int N0pad, int Dpad, int RS, const void *d_tiles, int ntiles) {
-    int HS = N0pad + Dpad, MP = 2 * Dpad;
+                    int N0pad, int HS, int MP, int RS, const void *d_tiles, int ntiles) {
     if (ntiles == 0) return HFX_OK;
     if (NC > 0x7fffffffLL / 4) return set_err(ctx, HFX_EUNSUPPORTED, "batch has too many columns for 32-bit TMA coordinates");
     int rc;
@@ -890,7 +981,6 @@ int launch_gemm1_tc(hfx_ctx *ctx, const __nv_bfloat16 *d_Ap_all, long long ap_ro
     p.HS = HS;
     p.MP = MP;
     p.N0pad = N0pad;
-    p.Dpad = Dpad;
     p.err = ctx->d_err;
     size_t smem = (size_t)G1_STAGES * G1_STAGE + 1024;
     auto kern = gemm1_kernel;

@@ -267,12 +267,11 @@ __global__ void transform_v_kernel(const double2 *v, double2 *VD, double2 *VB, c
 // Element (r, c) of the real embedding [[Ur, -Ui], [Ui, Ur]] of the
 // dense-block rows of U, the upper triangle of v_t with half its diagonal
 // (v_t = U + U^H for Hermitian v_t, so Z^H v_t Z = P' + P'^H with P' = Z^H U Z):
-// rows [Re D (Dpad) | Im D (Dpad)], columns [Re (N0pad + Dpad) | Im (N0pad +
-// Dpad)] (zero in the padding).  In the order [mu=0 | dense], the mu = 0
+// columns [Re (HS) | Im (HS)], each half the mu = 0 functions (N0pad) and the dense
+// ones (zero in the padding).  In the order [mu=0 | dense], the mu = 0
 // columns of the dense-block rows lie below the diagonal and are zero in U.
 __device__ __forceinline__ double ap_elem(const double2 *VD, int r, int c, int D, int naux, int N0, int N0pad,
-                                         int Dpad, int interleave) {
-    int HS = N0pad + Dpad;
+                                         int HS, int interleave) {
     // interleaved: row 2r real, 2r + 1 imaginary part of row r; else real rows
     // [0, D), imaginary rows [D, 2D)
     int rim = interleave ? (r & 1) : (r >= D), rr = interleave ? (r >> 1) : (rim ? r - D : r);
@@ -290,17 +289,17 @@ __device__ __forceinline__ double ap_elem(const double2 *VD, int r, int c, int D
 
 // Fixed-point slices of A' (one block per row; rows 2r and 2r + 1 the real and
 // imaginary parts of row r, or with a real v_t rows [0, D) real and [D, 2D)
-// imaginary; the rest of the 2 Dpad rows zero): exponent e_r with
+// imaginary; the rest of the MP rows zero): exponent e_r with
 // max_c |A'_rc| < 2^e_r, then the four slices of tc_ptx.cuh per element, stored
-// as BF16 planes [4][2 Dpad][RS] (the slice format of k_contract_tc.cu).
+// as BF16 planes [4][MP][RS] (the slice format of k_contract_tc.cu).
 __global__ void build_ap_kernel(const double2 *VD, __nv_bfloat16 *Ap, int *aexp, int D, int naux, int N0, int N0pad,
-                                int Dpad, int RS, int interleave) {
+                                int HS, int MP, int RS, int interleave) {
     int r = blockIdx.x;
-    long long plane = 2LL * Dpad * RS;
+    long long plane = (long long)MP * RS;
     __shared__ unsigned long long red[256];
     unsigned long long mx = 0;
     for (int c = threadIdx.x; c < RS; c += blockDim.x)
-        mx = max(mx, tc::abs_bits(ap_elem(VD, r, c, D, naux, N0, N0pad, Dpad, interleave)));
+        mx = max(mx, tc::abs_bits(ap_elem(VD, r, c, D, naux, N0, N0pad, HS, interleave)));
     red[threadIdx.x] = mx;
     __syncthreads();
     for (int st = blockDim.x / 2; st > 0; st >>= 1) {
@@ -311,7 +310,7 @@ __global__ void build_ap_kernel(const double2 *VD, __nv_bfloat16 *Ap, int *aexp,
     if (threadIdx.x == 0) aexp[r] = e;
     for (int c = threadIdx.x; c < RS; c += blockDim.x) {
         __nv_bfloat16 sl[tc::NPL];
-        tc::slice4(ap_elem(VD, r, c, D, naux, N0, N0pad, Dpad, interleave), e, sl);
+        tc::slice4(ap_elem(VD, r, c, D, naux, N0, N0pad, HS, interleave), e, sl);
         for (int i = 0; i < tc::NPL; ++i) Ap[i * plane + (long long)r * RS + c] = sl[i];
     }
 }
@@ -535,8 +534,8 @@ void launch_transform_v(const double2 *d_v, double2 *d_VD, double2 *d_VB, const 
 }
 
 void launch_build_ap(const double2 *d_VD, __nv_bfloat16 *d_Ap, int *d_aexp, int D, int naux, int N0, int N0pad,
-                     int Dpad, int RS, int interleave, cudaStream_t st) {
-    build_ap_kernel<<<2 * Dpad, 256, 0, st>>>(d_VD, d_Ap, d_aexp, D, naux, N0, N0pad, Dpad, RS, interleave);
+                     int HS, int MP, int RS, int interleave, cudaStream_t st) {
+    build_ap_kernel<<<MP, 256, 0, st>>>(d_VD, d_Ap, d_aexp, D, naux, N0, N0pad, HS, MP, RS, interleave);
 }
 
 void launch_check_coulomb(double2 *d_v, int naux, int zero_im, CoulombCheck *d_chk, cudaStream_t st) {

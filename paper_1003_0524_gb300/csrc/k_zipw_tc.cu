@@ -787,7 +787,7 @@ int zipw_tc_valid_nb(int nb) { return nb >= 8 && nb <= 64 && nb % 8 == 0; }
 int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, const char *dtab, const char *dscr,
                       __nv_bfloat16 *dTq, const PairDesc *d_pairs, const double2 *const *d_Tk, const int *d_nb,
                       double2 *d_Z, long long RSc, double2 *d_ZI, long long NCi, const QDesc *d_qd, int nq,
-                      long long maxcols, int max_nipw, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch) {
+                      long long maxcols, int max_nipw, bool transpose, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch) {
     if (!zb.ok || !bt.ok) return HFX_OK;
     cudaStream_t st = ctx->stream;
     int rc;
@@ -870,11 +870,11 @@ int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, co
     }
     if (rc_launch) return rc_launch;
     if ((rc = cuda_check(ctx, cudaGetLastError(), "zipw tensor-core kernel"))) return rc;
-    if (nq > 0 && maxcols > 0 && max_nipw > 0) {
+    if (transpose && nq > 0 && maxcols > 0 && max_nipw > 0) {
         const dim3 tg((unsigned)((maxcols + 31) / 32), (unsigned)((max_nipw + 31) / 32), (unsigned)nq);
         ipw_transpose_kernel<<<tg, 256, 0, st>>>(d_ZI, NCi, d_Z, RSc, ctx->nmt, d_qd);
     }
-    if (nlaunch) *nlaunch += 3;
+    if (nlaunch) *nlaunch += transpose ? 3 : 2;
     return cuda_check(ctx, cudaGetLastError(), "interstitial transpose");
 }
 
