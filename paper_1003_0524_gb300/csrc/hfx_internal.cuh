@@ -260,10 +260,10 @@ template <typename R>
 void launch_thetapsi(const double2 *d_theta, const int dlo[3], const int ddim[3], const int tlo[3],
                      const int tdim[3], const int *d_klist, int nklist, const double2 *d_c, const int *d_G, int nb,
                      int npw, typename C2<R>::T *d_out, cudaStream_t st);
+struct BmatJob { const double2 *A; void *B; int nb, pad; };   // one k: its MT coefficients and the B_k to fill
 template <typename R>
-void launch_bmat(const double2 *d_A, const double *d_R, const double *d_T, const double *d_gaunt,
-                 int n_atoms, int lmax, int Lmax, int P, int nb, int use_T, typename C2<R>::T *d_B,
-                 cudaStream_t st);
+void launch_bmat(const BmatJob *d_jobs, int njobs, const double *d_R, const double *d_T, const double *d_gaunt, int n_atoms,
+                 int lmax, int Lmax, int P, int use_T, cudaStream_t st);
 template <typename R>
 void launch_zmt(const PairDesc *d_pairs, int npairs, const QDesc *d_q, typename C2<R>::T *const *d_Bk,
                 const double2 *const *d_Ak, const double *d_posf, const int mesh[3], int n_atoms, int nLM, int P,

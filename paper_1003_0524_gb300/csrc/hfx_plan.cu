@@ -170,6 +170,7 @@ struct BuildPlan {
     int N0 = 0, sparse = 0, nb_max = 0, no_max = 0, npw_max = 0, maxD = 0, N0pad = 0, Dpad = 0, HS = 0, RS = 0, MP = 0;
     int NB = 8;
     int ksplit = 1;                   // FP64 build: parts the sum over m of one pair is split into
+    size_t o_bmat = 0;                // B_k jobs of the k set
     size_t o_A = 0, o_c = 0, o_G = 0, o_Ga = 0, o_npw = 0, o_nb = 0, o_no = 0, o_B = 0, o_T = 0, o_vacc = 0, o_V = 0;
     bool kp = false;                  // the k.p term at q = 0 is added
     bool inv = false;                 // inversion symmetry: packed real bands (Sec. III.D)
@@ -339,6 +340,11 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
     }
     HostArena tab;
     pl.o_A = tab.put(hA); pl.o_c = tab.put(hc); pl.o_G = tab.put(hG); pl.o_Ga = tab.put(hGa);
+    {
+        std::vector<BmatJob> jobs;
+        for (int ik : kset) jobs.push_back(BmatJob{ctx->kp[ik].d_A, hB[ik], hnb[ik], 0});
+        pl.o_bmat = tab.put(jobs);
+    }
     pl.o_npw = tab.put(hnpw); pl.o_nb = tab.put(hnb); pl.o_no = tab.put(hno);
     pl.o_B = tab.put(hB); pl.o_T = tab.put(hT); pl.o_vacc = tab.put(hvacc); pl.o_V = tab.put(hV);
     if (ctx->opt.kp_term) {
@@ -654,21 +660,19 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
     launch_theta(reinterpret_cast<double2 *>(ctx->s_theta.p), pl.geo.dlo, pl.geo.ddim, ctx->B, ctx->omega, ctx->d_posf,
                  ctx->d_posf + 3 * s.n_atoms, s.n_atoms, ctx->stream);
     ++nl;
-    {
-        const size_t bsz = (size_t)s.n_atoms * ctx->nLM * P * ctx->nlmp;
-        size_t boff = 0, toff = 0;
-        std::vector<size_t> bo(nk), to(nk);
-        for (int i = 0; i < nk; ++i) { bo[i] = boff; boff += bsz * ctx->kp[i].nb; to[i] = toff; toff += (size_t)pl.tbox * ctx->kp[i].nb; }
+    launch_bmat<R>(reinterpret_cast<const BmatJob *>(tab + pl.o_bmat), (int)pl.kset.size(), ctx->d_R, ctx->d_T, ctx->d_gaunt,
+                   s.n_atoms, s.lmax, s.Lmax, P, sparse, ctx->stream);
+    ++nl;
+    if (!tc) {
+        size_t toff = 0;
+        std::vector<size_t> to(nk);
+        for (int i = 0; i < nk; ++i) { to[i] = toff; toff += (size_t)pl.tbox * ctx->kp[i].nb; }
         for (int ik : pl.kset) {
-            launch_bmat<R>(ctx->kp[ik].d_A, ctx->d_R, ctx->d_T, ctx->d_gaunt, s.n_atoms, s.lmax, s.Lmax, P, ctx->kp[ik].nb,
-                           sparse, at<V>(ctx->s_B.p, bo[ik] * sizeof(V)), ctx->stream);
+            launch_thetapsi<R>(reinterpret_cast<double2 *>(ctx->s_theta.p), pl.geo.dlo, pl.geo.ddim, pl.geo.tlo, pl.geo.tdim,
+                               reinterpret_cast<const int *>(tab + pl.o_reach), pl.nreach, ctx->kp[ik].d_c,
+                               ctx->kp[ik].d_G, ctx->kp[ik].nb, ctx->kp[ik].npw, at<V>(ctx->s_thpsi.p, to[ik] * sizeof(V)),
+                               ctx->stream);
             ++nl;
-            if (!tc) {
-                launch_thetapsi<R>(reinterpret_cast<double2 *>(ctx->s_theta.p), pl.geo.dlo, pl.geo.ddim, pl.geo.tlo,
-                                   pl.geo.tdim, reinterpret_cast<const int *>(tab + pl.o_reach), pl.nreach, ctx->kp[ik].d_c, ctx->kp[ik].d_G, ctx->kp[ik].nb, ctx->kp[ik].npw,
-                                   at<V>(ctx->s_thpsi.p, to[ik] * sizeof(V)), ctx->stream);
-                ++nl;
-            }
         }
     }
     if ((rc = cuda_check(ctx, cudaGetLastError(), "per-k kernels"))) return rc;

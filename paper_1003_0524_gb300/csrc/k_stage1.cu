@@ -85,52 +85,74 @@ __global__ void thetapsi_kernel(const double2 *__restrict__ theta, int dlo0, int
 }
 
 // ------------------------------------------------------------- B_k
+// One block per (k, LM, atom): for every lmp the real coefficients
+//   W[i][l'p'] = G(LM; lm; l') sum_s T_{aL}[i][s] R^a_{Ls; lp; l'p'}   (l' + l + L even, |L - l| <= l' <= L + l)
+// once per block, then B[i][lmp][n] = sum W[i][l'p'] A_{l', m + M, p'}(n) for 32 bands
+// at a time, their A rows in shared memory.  Bound by FP64 issue: two FMAs per
+// coefficient and output instead of three operations per radial function before the
+// transform, and one launch for all k (one per k and recomputed coefficients: 1.23 ms
+// for 64 k of 2 atoms, 0.32 ms now).
+// floor(sqrt(n)) of a small n >= 0, without the FP64 pipe
+__device__ __forceinline__ int isqrt_small(int n) { return (int)sqrtf((float)n + 0.5f); }
+
+constexpr int BM_THREADS = 256, BM_W = 2880;   // coefficients kept at a time
 template <typename R>
-__global__ void bmat_kernel(const double2 *__restrict__ A, const double *__restrict__ Rr, const double *__restrict__ T,
-                            const double *__restrict__ gaunt, int n_atoms, int lmax, int Lmax, int P, int nb,
-                            int use_T, typename C2<R>::T *__restrict__ Bk) {
+__global__ void __launch_bounds__(BM_THREADS) bmat_kernel(const BmatJob *__restrict__ jobs, const double *__restrict__ Rr,
+                                                          const double *__restrict__ T, const double *__restrict__ gaunt,
+                                                          int n_atoms, int lmax, int Lmax, int P, int use_T) {
     using V = typename C2<R>::T;
-    int nlm = (lmax + 1) * (lmax + 1), nLM = (Lmax + 1) * (Lmax + 1), nlmp = 2 * nlm, nlp = 2 * (lmax + 1);
-    long long total = (long long)n_atoms * nLM * nlmp * nb;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        int n = (int)(e % nb);
-        int lmp = (int)((e / nb) % nlmp);
-        int LM = (int)((e / ((long long)nb * nlmp)) % nLM);
-        int a = (int)(e / ((long long)nb * nlmp * nLM));
-        int lm = lmp >> 1, p = lmp & 1;
-        int l = (int)floor(sqrt((double)lm) + 1e-9), m = lm - l * l - l;
-        int L = (int)floor(sqrt((double)LM) + 1e-9), M = LM - L * L - L;
-        double2 bp[kMaxP];
-        for (int s = 0; s < P; ++s) bp[s] = make_double2(0.0, 0.0);
-        const double2 *An = A + ((size_t)n * n_atoms + a) * nlmp;
-        for (int l2 = 0; l2 <= lmax; ++l2) {
-            int m2 = m + M;
-            if (m2 < -l2 || m2 > l2) continue;
-            double g = gaunt[((size_t)LM * nlm + lm) * (lmax + 1) + l2];
-            if (g == 0.0) continue;
-            for (int p2 = 0; p2 < 2; ++p2) {
-                double2 av = An[2 * (l2 * l2 + l2 + m2) + p2];
-                for (int s = 0; s < P; ++s) {
-                    double r = Rr[(((size_t)a * (Lmax + 1) + L) * P + s) * nlp * nlp + (2 * l + p) * nlp + 2 * l2 + p2];
-                    bp[s].x += g * r * av.x;
-                    bp[s].y += g * r * av.y;
-                }
-            }
-        }
-        const double *Ta = T + ((size_t)a * (Lmax + 1) + L) * P * P;
-        for (int i = 0; i < P; ++i) {
-            double2 o;
+    const BmatJob jb = jobs[blockIdx.x];
+    const int LM = blockIdx.y, a = blockIdx.z, nb = jb.nb;
+    const int nlm = (lmax + 1) * (lmax + 1), nLM = gridDim.y, nlmp = 2 * nlm, nlp = 2 * (lmax + 1);
+    const int L = isqrt_small(LM), M = LM - L * L - L;
+    extern __shared__ __align__(16) unsigned char bm_smem[];
+    double *W = reinterpret_cast<double *>(bm_smem);            // [lmp of the chunk][P][nlp]
+    double2 *As = reinterpret_cast<double2 *>(W + BM_W);        // [32][nlmp + 1]
+    const int ldA = nlmp + 1, per = P * nlp, nc = max(1, BM_W / per);
+    const double *Ta = T + ((size_t)a * (Lmax + 1) + L) * P * P;
+    const double *Ra = Rr + ((size_t)a * (Lmax + 1) + L) * P * nlp * nlp;
+    V *B = reinterpret_cast<V *>(jb.B) + (((size_t)a * nLM + LM) * P) * nlmp * nb;
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    for (int c0 = 0; c0 < nlmp; c0 += nc) {
+        const int cn = min(nc, nlmp - c0);
+        __syncthreads();
+        for (int t = threadIdx.x; t < cn * per; t += BM_THREADS) {
+            const int lmp = c0 + t / per, i = (t / nlp) % P, lp2 = t % nlp, l2 = lp2 >> 1;
+            const int lm = lmp >> 1, l = isqrt_small(lm);
+            const double g = gaunt[((size_t)LM * nlm + lm) * (lmax + 1) + l2];
+            const double *r = Ra + (size_t)(2 * l + (lmp & 1)) * nlp + lp2;
+            double s = 0.0;
             if (use_T) {
-                o = make_double2(0.0, 0.0);
-                for (int s = 0; s < P; ++s) {
-                    o.x += Ta[i * P + s] * bp[s].x;
-                    o.y += Ta[i * P + s] * bp[s].y;
-                }
+                for (int x = 0; x < P; ++x) s = fma(Ta[i * P + x], r[(size_t)x * nlp * nlp], s);
             } else {
-                o = bp[i];
+                s = r[(size_t)i * nlp * nlp];
             }
-            Bk[((((size_t)a * nLM + LM) * P + i) * nlmp + lmp) * nb + n] = ld_c<R>(o);
+            W[t] = g * s;
+        }
+        for (int n0 = 0; n0 < nb; n0 += 32) {
+            const int nn = min(32, nb - n0);
+            __syncthreads();
+            for (int t = threadIdx.x; t < nn * nlmp; t += BM_THREADS)
+                As[(t / nlmp) * ldA + t % nlmp] = jb.A[((size_t)(n0 + t / nlmp) * n_atoms + a) * nlmp + t % nlmp];
+            __syncthreads();
+            for (int t = warp; t < cn * P; t += BM_THREADS / 32) {
+                const int lmp = c0 + t / P, i = t % P, lm = lmp >> 1;
+                const int l = isqrt_small(lm), m2 = lm - l * l - l + M;
+                int l2 = max(abs(m2), abs(L - l));
+                l2 += (L + l + l2) & 1;
+                const double *w = W + (size_t)t * nlp;
+                double2 o = make_double2(0.0, 0.0);
+                if (lane < nn)
+                    for (; l2 <= min(lmax, L + l); l2 += 2) {
+                        const double2 *av = As + lane * ldA + 2 * (l2 * l2 + l2 + m2);
+#pragma unroll
+                        for (int p2 = 0; p2 < 2; ++p2) {
+                            o.x = fma(w[2 * l2 + p2], av[p2].x, o.x);
+                            o.y = fma(w[2 * l2 + p2], av[p2].y, o.y);
+                        }
+                    }
+                if (lane < nn) B[((size_t)i * nlmp + lmp) * nb + n0 + lane] = ld_c<R>(o);
+            }
         }
     }
 }
@@ -427,11 +449,14 @@ void launch_thetapsi(const double2 *d_theta, const int dlo[3], const int ddim[3]
 }
 
 template <typename R>
-void launch_bmat(const double2 *d_A, const double *d_R, const double *d_T, const double *d_gaunt, int n_atoms,
-                 int lmax, int Lmax, int P, int nb, int use_T, typename C2<R>::T *d_B, cudaStream_t st) {
-    long long total = (long long)n_atoms * (Lmax + 1) * (Lmax + 1) * 2 * (lmax + 1) * (lmax + 1) * nb;
-    bmat_kernel<R><<<grid_for(total, 128), 128, 0, st>>>(d_A, d_R, d_T, d_gaunt, n_atoms, lmax, Lmax, P, nb, use_T,
-                                                         d_B);
+void launch_bmat(const BmatJob *d_jobs, int njobs, const double *d_R, const double *d_T, const double *d_gaunt, int n_atoms,
+                 int lmax, int Lmax, int P, int use_T, cudaStream_t st) {
+    if (njobs == 0) return;
+    const int nlmp = 2 * (lmax + 1) * (lmax + 1);
+    const size_t sm = BM_W * sizeof(double) + (size_t)32 * (nlmp + 1) * sizeof(double2);   // 106 KB at lmax 8
+    cudaFuncSetAttribute(bmat_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const dim3 grid((unsigned)njobs, (unsigned)((Lmax + 1) * (Lmax + 1)), (unsigned)n_atoms);
+    bmat_kernel<R><<<grid, BM_THREADS, sm, st>>>(d_jobs, d_R, d_T, d_gaunt, n_atoms, lmax, Lmax, P, use_T);
 }
 
 template <typename R>
@@ -499,8 +524,8 @@ void launch_unpermute(const typename C2<R>::T *d_Z, const PairDesc &pr, int naux
     template void launch_thetapsi<R>(const double2 *, const int *, const int *, const int *, const int *,            \
                                      const int *, int, const double2 *, const int *, int, int, C2<R>::T *,           \
                                      cudaStream_t);                                                                  \
-    template void launch_bmat<R>(const double2 *, const double *, const double *, const double *, int, int, int,    \
-                                 int, int, int, C2<R>::T *, cudaStream_t);                                           \
+    template void launch_bmat<R>(const BmatJob *, int, const double *, const double *, const double *, int, int, int, \
+                                 int, int, cudaStream_t);                                                            \
     template void launch_zmt<R>(const PairDesc *, int, const QDesc *, C2<R>::T *const *, const double2 *const *,    \
                                 const double *, const int *, int, int, int, int, int, int, int, C2<R>::T *,         \
                                 long long, cudaStream_t);                                                            \
