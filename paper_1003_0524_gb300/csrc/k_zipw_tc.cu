@@ -507,13 +507,20 @@ __global__ void __launch_bounds__(256) ipw_transpose_kernel(const double2 *__res
     }
 }
 
-// band block: a multiple of 8 (the output width 2 NB is a multiple of 16),
-// at most 40 (two pipeline stages in shared memory), fewest padded bands
+// Band block: a multiple of 8 (the output width 2 NB is a multiple of 16) up to 64, the
+// one with the least padded bands times the time per padded band.  A narrow block reads
+// the 128 rows of A from shared memory for fewer columns; measured per band against 64
+// (2 atoms, 40 and 32 to 48 bands; 5 atoms, 120; 10 atoms, 250): 8: 3.1, 16: 1.74, 24:
+// 1.33, 32: 1.19, 40: 1.04 to 1.12, 48: 1.08, 56: 1.02.  (The least padding among 8 to
+// 40 took 24 for 48 bands, 70.1 ms against 57.3 with 48, and 32 for 250 bands, 7.5 ms
+// against 6.6 with 64.)
 int pick_nb(int nb_max) {
-    int best = 8, best_tot = 1 << 30;
-    for (int nb = 8; nb <= 40; nb += 8) {
-        int tot = (nb_max + nb - 1) / nb * nb;
-        if (tot < best_tot || (tot == best_tot && nb > best)) { best = nb; best_tot = tot; }
+    static const double per_band[8] = {3.1, 1.74, 1.33, 1.19, 1.06, 1.08, 1.02, 1.0};
+    int best = 8;
+    double cost = 1e300;
+    for (int nb = 8; nb <= 64; nb += 8) {
+        const double c = per_band[nb / 8 - 1] * ((nb_max + nb - 1) / nb * nb);
+        if (c <= cost) { best = nb; cost = c; }
     }
     return best;
 }
