@@ -626,9 +626,27 @@ int prepare_coulomb(hfx_ctx *ctx) {
     dfree(d_mx);
     ctx->sparse_used = sparse;
     ctx->N0 = sparse ? ctx->nch * (P - 1) : 0;
+    ctx->mod_used = false;
     if (ctx->opt.precision == HFX_PREC_SLICED) {
         int maxD = 0;
         for (auto &q : ctx->qp) maxD = std::max(maxD, ctx->nmt + q.nipw - ctx->N0);
+        if (!ctx->opt.inversion && apply_mod_usable(maxD)) {
+            const ModSizes z = apply_mod_sizes(maxD);
+            if ((rc = scratch_reserve(ctx, ctx->s_ap, z.u_elems * ctx->nk * sizeof(__nv_bfloat16))) ||
+                (rc = scratch_reserve(ctx, ctx->s_aexp, (size_t)z.Dp * ctx->nk * sizeof(int))))
+                return rc;
+            for (int iq = 0; iq < ctx->nk; ++iq) {
+                const int naux = ctx->nmt + ctx->qp[iq].nipw;
+                if ((rc = apply_mod_prepare_u(ctx, ctx->qp[iq].d_VD, reinterpret_cast<__nv_bfloat16 *>(ctx->s_ap.p) + z.u_elems * iq,
+                                              reinterpret_cast<int *>(ctx->s_aexp.p) + (size_t)z.Dp * iq, naux - ctx->N0, naux,
+                                              ctx->N0, z)))
+                    return rc;
+            }
+            if ((rc = sync(ctx))) return rc;
+            ctx->mod_used = true;
+            ctx->coulomb_dirty = false;
+            return HFX_OK;
+        }
         int N0pad = (int)rup(ctx->N0, 64), Dpad = (int)rup(maxD, 128);
         int HS = slice_half(N0pad, maxD), RS = 2 * HS, MP = 2 * Dpad;
         size_t per = (size_t)4 * MP * RS;

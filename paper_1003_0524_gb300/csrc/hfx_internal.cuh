@@ -174,6 +174,7 @@ struct hfx_ctx {
 
     bool coulomb_dirty = true;   // transform must be redone
     bool sparse_used = false;
+    bool mod_used = false;       // the Coulomb apply runs on residues (s_ap, s_aexp hold those of U)
     int N0 = 0;                  // mu=0 rows (sparse) or 0 (dense)
     double q0_bracket = 0.0;
     bool q0_valid = false;
@@ -319,7 +320,7 @@ int launch_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long NCi, const doubl
 // triangle; the Hermitian split passes null.)
 template <typename V>
 void launch_block_y(const QDesc *d_q, int nq, const double2 *const *d_VB, const double2 *const *d_VD, const V *d_Z,
-                    double2 *d_Y, long long RSc, int P, int N0, long long maxcols, cudaStream_t st);
+                    double2 *d_Y, long long RSc, long long ldY, int P, int N0, long long maxcols, cudaStream_t st);
 bool block_y_couples(int P, int N0);
 // Half width of the slice rows: the mu = 0 rows (N0pad) and the dense rows, padded to a
 // multiple of 128.  (64 would save 8 % of the planes of the 2-atom workload, but its
@@ -334,6 +335,26 @@ int gemm1_tiles(const QDesc *h_q, int nq, int N0pad, bool real_v, std::vector<un
 int launch_gemm1_tc(hfx_ctx *ctx, const __nv_bfloat16 *d_Ap_all, long long ap_rows, const int *d_aexp, const QDesc *d_q,
                     const __nv_bfloat16 *d_ZS, const int *d_zexp, double2 *d_Y, long long RSc, long long NC, int N0,
                     int N0pad, int HS, int MP, int RS, const void *d_tiles, int ntiles);
+// ------------------------------------------------------------ the apply of large dense blocks (k_apply_mod.cu)
+struct ModSizes {            // of the largest dense block
+    int Kp = 0, Dp = 0;      // K (64) and rows of U (256) padded
+    size_t u_elems = 0;      // BF16 elements of the residues of one U
+    size_t col_bytes = 0;    // bytes of the residues of one column of Z or Y'
+};
+bool apply_mod_usable(int maxD);
+ModSizes apply_mod_sizes(int maxD);
+int apply_mod_prepare_u(hfx_ctx *ctx, const double2 *d_VD, __nv_bfloat16 *d_UR, int *d_uexp, int D, int naux, int N0,
+                        const ModSizes &z);
+int apply_mod_tiles(const QDesc *h_q, int nq, std::vector<unsigned char> &out);
+int apply_mod_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long sg, long long sc, const double2 *d_Z, long long RSc,
+                      const QDesc *d_q, int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
+                      const ModSizes &z, __nv_bfloat16 *d_ZS, __nv_bfloat16 *d_ZR, int *d_xexp, int *d_zexp);
+int apply_mod_run(hfx_ctx *ctx, const __nv_bfloat16 *d_UR_all, int nk, const __nv_bfloat16 *d_ZR, short *d_YR, long long NC,
+                  const ModSizes &z, const void *d_tiles, int nplane);
+int apply_mod_slice_y(hfx_ctx *ctx, const short *d_YR, const double2 *d_Y0, const QDesc *d_q, int nq, const int *d_uexp,
+                      const int *d_zexp, long long NC, long long maxcols, int N0, int N0pad, int HS, int RS, const ModSizes &z,
+                      __nv_bfloat16 *d_YS, int *d_yexp);
+
 // real_form: the Z^H Y tiles of the inversion-symmetric path (only Re P', two
 // row blocks per tile; band blocks of 16, 32, 48 or 64, see gemm2_real_form)
 int gemm2_tiles(const PairDesc *h_pairs, int npairs, int NB, bool real_form, std::vector<unsigned char> &out);

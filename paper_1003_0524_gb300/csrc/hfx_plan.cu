@@ -154,6 +154,8 @@ struct BatchPlan {
     int nklist = 0;
     size_t o_pairs = 0, o_qd = 0, o_kpair = 0, o_praw = 0, o_klist = 0, o_kstart = 0, o_klp = 0, o_vb = 0, o_vd = 0;
     size_t o_zg1 = 0, o_zg2 = 0, o_g1t = 0, o_g2t = 0;
+    size_t o_mq = 0;                  // modular apply: the tiles of one residue plane
+    int n_mt = 0;
     int n_g1t = 0, n_g2t = 0, maxM1 = 0, maxN1 = 0, mx2 = 0;
     ZipwBatch zipw;
     ZmtBatch zmt;
@@ -169,6 +171,9 @@ struct BuildPlan {
     long long tbox = 0, dbox = 0, RSc = 0;
     int N0 = 0, sparse = 0, nb_max = 0, no_max = 0, npw_max = 0, maxD = 0, N0pad = 0, Dpad = 0, HS = 0, RS = 0, MP = 0;
     int NB = 8;
+    long long ncol_max = 1;           // columns of the largest batch
+    bool mod = false;                 // the apply runs on residues (k_apply_mod.cu)
+    ModSizes ms;
     int ksplit = 1;                   // FP64 build: parts the sum over m of one pair is split into
     size_t o_bmat = 0;                // B_k jobs of the k set
     size_t o_A = 0, o_c = 0, o_G = 0, o_Ga = 0, o_npw = 0, o_nb = 0, o_no = 0, o_B = 0, o_T = 0, o_vacc = 0, o_V = 0;
@@ -216,7 +221,7 @@ namespace {
 
 Scratch *build_scratch(hfx_ctx *ctx, int i) {
     Scratch *all[] = {&ctx->s_theta, &ctx->s_thpsi, &ctx->s_B,   &ctx->s_zc,   &ctx->s_zs,  &ctx->s_ys,  &ctx->s_y64,
-                      &ctx->s_praw,  &ctx->s_vacc,  &ctx->s_xexp, &ctx->s_zipw, &ctx->s_cgT, &ctx->s_cgZ};
+                      &ctx->s_praw,  &ctx->s_vacc,  &ctx->s_pairs, &ctx->s_xexp, &ctx->s_zipw, &ctx->s_cgT, &ctx->s_cgZ};
     return i < (int)(sizeof(all) / sizeof(all[0])) ? all[i] : nullptr;
 }
 
@@ -239,6 +244,7 @@ uint64_t plan_signature(hfx_ctx *ctx, const std::vector<int> &kset) {
     h.val(ctx->opt.q0_term);
     h.val(ctx->q0_bracket);
     h.val(ctx->sparse_used);
+    h.val(ctx->mod_used);
     h.val(ctx->N0);
     for (auto &k : ctx->kp) { h.val(k.d_G); h.val(k.d_c); h.val(k.d_A); h.val(k.nb); h.val(k.no); h.val(k.npw); }
     for (auto &q : ctx->qp) { h.val(q.d_G); h.val(q.d_VD); h.val(q.d_VB); h.val(q.nipw); }
@@ -279,6 +285,15 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
     pl.HS = slice_half(pl.N0pad, pl.maxD);
     pl.RS = 2 * pl.HS;
     pl.MP = 2 * pl.Dpad;
+    pl.mod = tc && ctx->mod_used;
+    if (pl.mod) pl.ms = apply_mod_sizes(pl.maxD);
+    // bytes per column of the buffers that change their contents within a batch: Z and
+    // the interstitial plane (for the modular apply in one allocation, where the residues
+    // of Y' replace both), the residues of Z and then the digits of Y'
+    const size_t y_bytes = pl.mod ? 0 : (size_t)pl.RSc * sizeof(double2);
+    const size_t z_bytes = pl.mod ? std::max<size_t>((size_t)2 * pl.RSc * sizeof(double2), pl.ms.col_bytes)
+                                  : (size_t)pl.RSc * sizeof(V);
+    const size_t ys_bytes = std::max<size_t>((size_t)4 * pl.RS * sizeof(__nv_bfloat16), pl.mod ? pl.ms.col_bytes : 0);
     const long long RSc = pl.RSc;
     pl.NB = gemm2_check_nb(ctx->opt.tile_nb_zhy) ? ctx->opt.tile_nb_zhy : pick_nb_zhy(pl.nb_max);
     const int NB = pl.NB;
@@ -394,8 +409,9 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         const long long nc = (long long)hnom[ikp] * hnb[ik];
         size_t praw = tc ? (size_t)((hnb[ik] + NB - 1) / NB) * ((hnb[ik] + NB - 1) / NB) * (2 * NB) * (2 * NB) * sizeof(double)
                          : (size_t)ksplit * hnb[ik] * hnb[ik] * sizeof(double2);
-        size_t b = (size_t)nc * RSc * sizeof(V) + praw + (size_t)nc * RSc * sizeof(double2);
-        if (tc) b += (size_t)2 * 4 * nc * pl.RS * sizeof(__nv_bfloat16) + 2 * nc * sizeof(int);
+        size_t b = (size_t)nc * z_bytes + praw + nc * y_bytes;
+        if (tc) b += nc * ((size_t)4 * pl.RS * sizeof(__nv_bfloat16) + ys_bytes + 3 * sizeof(int));
+        if (pl.mod) b += (size_t)nc * N0 * sizeof(double2);
         return b;
     };
     std::vector<std::vector<std::pair<int, int>>> groups;   // (ik, iq) per batch, k-major
@@ -507,17 +523,20 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
 
     // ---- scratch of the batches and of the tensor-core stages
     const size_t ncol_max = (size_t)std::max<long long>(1, max_ncols);
-    if ((rc = scratch_reserve(ctx, ctx->s_zc, ncol_max * RSc * sizeof(V))) ||
+    pl.ncol_max = (long long)ncol_max;
+    if ((rc = scratch_reserve(ctx, ctx->s_zc, ncol_max * z_bytes)) ||
         (rc = scratch_reserve(ctx, ctx->s_praw, (size_t)std::max<long long>(1, max_praw) * sizeof(double))) ||
-        (rc = scratch_reserve(ctx, ctx->s_y64, ncol_max * RSc * sizeof(double2))))
+        (rc = scratch_reserve(ctx, ctx->s_y64, ncol_max * y_bytes)))
         return rc;
+    // the mu = 0 rows of Y' (FP64), which have no place among the residues
+    if (pl.mod && (rc = scratch_reserve(ctx, ctx->s_pairs, std::max<size_t>(ncol_max * N0 * sizeof(double2), 256)))) return rc;
     if (tc) {
         Layout zl;
         zl.place(pl.zipw.scratch_bytes);
         pl.zipw_tq_off = zl.place(std::max<size_t>(max_tq, 256));
         if ((rc = scratch_reserve(ctx, ctx->s_zs, (size_t)4 * ncol_max * pl.RS * sizeof(__nv_bfloat16))) ||
-            (rc = scratch_reserve(ctx, ctx->s_ys, (size_t)4 * ncol_max * pl.RS * sizeof(__nv_bfloat16))) ||
-            (rc = scratch_reserve(ctx, ctx->s_xexp, (size_t)2 * ncol_max * sizeof(int))) ||
+            (rc = scratch_reserve(ctx, ctx->s_ys, ncol_max * ys_bytes)) ||
+            (rc = scratch_reserve(ctx, ctx->s_xexp, (size_t)3 * ncol_max * sizeof(int))) ||
             (rc = scratch_reserve(ctx, ctx->s_cgT, std::max<size_t>(pl.tp.scratch_bytes, 256))) ||
             (rc = scratch_reserve(ctx, ctx->s_cgZ, std::max<size_t>(pl.zmt.scratch_bytes, 256))) ||
             (rc = scratch_reserve(ctx, ctx->s_zipw, zl.off)))
@@ -573,7 +592,14 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         if (tc) {
             if ((rc = zmt_tc_plan_batch(ctx, pl.zmt, bt.pairs, RSc, tab, bt.zmt))) return rc;
             std::vector<unsigned char> t1, t2;
-            bt.n_g1t = gemm1_tiles(bt.qd.data(), nq, pl.N0pad, pl.inv, t1);
+            if (pl.mod) {
+                std::vector<unsigned char> tm;
+                if ((bt.n_mt = apply_mod_tiles(bt.qd.data(), nq, tm)) < 0)
+                    return set_err(ctx, HFX_EUNSUPPORTED, "apply: too many tiles in one batch");
+                bt.o_mq = tab.put(tm);
+            } else {
+                bt.n_g1t = gemm1_tiles(bt.qd.data(), nq, pl.N0pad, pl.inv, t1);
+            }
             bt.n_g2t = gemm2_tiles(bt.pairs.data(), npairs, NB, pl.inv && gemm2_real_form(NB), t2);
             bt.o_g1t = tab.put(t1);
             bt.o_g2t = tab.put(t2);
@@ -694,6 +720,8 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
 
     V *Zc = reinterpret_cast<V *>(ctx->s_zc.p);
     double *praw = reinterpret_cast<double *>(ctx->s_praw.p);
+    // the interstitial plane, later Y' in FP64
+    double2 *Yd = pl.mod ? reinterpret_cast<double2 *>(Zc) + pl.ncol_max * RSc : reinterpret_cast<double2 *>(ctx->s_y64.p);
     for (BatchPlan &bt : pl.batches) {
         const int npairs = (int)bt.pairs.size(), nq = (int)bt.qs.size();
         const PairDesc *d_pairs = reinterpret_cast<const PairDesc *>(tab + bt.o_pairs);
@@ -724,7 +752,7 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
                                         at<__nv_bfloat16>(ctx->s_zipw.p, pl.zipw_tq_off), d_pairs,
                                         reinterpret_cast<const double2 *const *>(tab + pl.o_T),
                                         reinterpret_cast<const int *>(tab + pl.o_nb), reinterpret_cast<double2 *>(Zc), RSc,
-                                        reinterpret_cast<double2 *>(ctx->s_y64.p), bt.ncols, d_qd, nq, bt.maxcols, max_nipw, z_whole,
+                                        Yd, bt.ncols, d_qd, nq, bt.maxcols, max_nipw, z_whole,
                                         bt.ev[2], bt.ev[3], &nl)))
                 return rc;
         } else {
@@ -771,9 +799,20 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
         // ---- contraction
         if (tc) {
             __nv_bfloat16 *ZS = reinterpret_cast<__nv_bfloat16 *>(ctx->s_zs.p), *YS = reinterpret_cast<__nv_bfloat16 *>(ctx->s_ys.p);
-            double2 *Yd = reinterpret_cast<double2 *>(ctx->s_y64.p);
             int *zexp = reinterpret_cast<int *>(ctx->s_xexp.p), *yexp = zexp + bt.ncols;
-            if (z_whole || !bt.zipw.ok) {
+            int *mexp = yexp + bt.ncols;   // powers of two of the residues of Z
+            // the interstitial rows: in the interstitial kernel's plane, or in Z
+            const bool in_z = z_whole || !bt.zipw.ok;
+            double2 *Y0 = reinterpret_cast<double2 *>(ctx->s_pairs.p);   // modular apply: mu = 0 rows of Y'
+            if (pl.mod) {
+                // (before the apply, which takes the place of Z)
+                launch_block_y<V>(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb), nullptr, Zc, Y0, RSc, N0,
+                                  P, N0, bt.maxcols, ctx->stream);
+                const double2 *Zd = reinterpret_cast<const double2 *>(Zc);
+                if ((rc = apply_mod_slice_z(ctx, in_z ? Zd + nmt : Yd, in_z ? 1 : bt.ncols, in_z ? RSc : 1, Zd, RSc, d_qd, nq,
+                                            bt.ncols, bt.maxcols, nmt, N0, pl.N0pad, pl.HS, pl.RS, pl.ms, ZS, YS, zexp, mexp)))
+                    return rc;
+            } else if (in_z) {
                 launch_slice_cols<V>(Zc, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.HS, pl.RS, ZS, zexp, ctx->stream);
                 if ((rc = cuda_check(ctx, cudaGetLastError(), "slice kernels"))) return rc;
             } else if ((rc = launch_slice_z(ctx, Yd, bt.ncols, reinterpret_cast<double2 *>(Zc), RSc, d_qd, nq, bt.ncols,
@@ -784,15 +823,27 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             // Y' = U Z with U the upper triangle of v_t (half diagonal): the dense
             // rows on the tensor cores, the mu = 0 rows in the channel-block kernel;
             // the q reduction adds P' + P'^H for P' = Z^H Y'
-            if ((rc = launch_gemm1_tc(ctx, reinterpret_cast<const __nv_bfloat16 *>(ctx->s_ap.p), (long long)nk * 4 * pl.MP,
-                                      reinterpret_cast<const int *>(ctx->s_aexp.p), d_qd, ZS, zexp, Yd, RSc, bt.ncols, N0,
-                                      pl.N0pad, pl.HS, pl.MP, pl.RS, tab + bt.o_g1t, bt.n_g1t)))
-                return rc;
+            if (pl.mod)
+                rc = apply_mod_run(ctx, reinterpret_cast<const __nv_bfloat16 *>(ctx->s_ap.p), nk, YS,
+                                   reinterpret_cast<short *>(Zc), bt.ncols, pl.ms, tab + bt.o_mq, bt.n_mt);
+            else
+                rc = launch_gemm1_tc(ctx, reinterpret_cast<const __nv_bfloat16 *>(ctx->s_ap.p), (long long)nk * 4 * pl.MP,
+                                     reinterpret_cast<const int *>(ctx->s_aexp.p), d_qd, ZS, zexp, Yd, RSc, bt.ncols, N0,
+                                     pl.N0pad, pl.HS, pl.MP, pl.RS, tab + bt.o_g1t, bt.n_g1t);
+            if (rc) return rc;
             rec(ctx, bt.ev[7]);
-            launch_block_y<V>(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb), nullptr, Zc, Yd, RSc, P,
-                              N0, bt.maxcols, ctx->stream);
-            launch_slice_cols<double2>(Yd, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.HS, pl.RS, YS, yexp,
-                                       ctx->stream);
+            if (!pl.mod)
+                launch_block_y<V>(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb), nullptr, Zc, Yd, RSc, RSc,
+                                  P, N0, bt.maxcols, ctx->stream);
+            if (pl.mod) {
+                if ((rc = apply_mod_slice_y(ctx, reinterpret_cast<const short *>(Zc), Y0, d_qd, nq,
+                                            reinterpret_cast<const int *>(ctx->s_aexp.p), mexp, bt.ncols, bt.maxcols, N0,
+                                            pl.N0pad, pl.HS, pl.RS, pl.ms, YS, yexp)))
+                    return rc;
+            } else {
+                launch_slice_cols<double2>(Yd, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.HS, pl.RS, YS, yexp,
+                                           ctx->stream);
+            }
             rec(ctx, bt.ev[8]);
             if ((rc = launch_gemm2_tc(ctx, ZS, YS, zexp, yexp, bt.ncols, pl.RS, pl.HS, pl.N0pad, d_pairs, d_qd, pl.NB,
                                       d_praw_off, praw, tab + bt.o_g2t, bt.n_g2t, fail_wait,
@@ -802,7 +853,6 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             rec(ctx, bt.ev[9]);
             nl += 5;
         } else {
-            double2 *Yd = reinterpret_cast<double2 *>(ctx->s_y64.p);
             rec(ctx, bt.ev[6]);
             launch_zgemm64(reinterpret_cast<const ZGemmBatch *>(tab + bt.o_zg1), nq, bt.maxM1, bt.maxN1, ctx->stream);
             rec(ctx, bt.ev[7]);

@@ -195,7 +195,7 @@ __device__ __forceinline__ double upper_weight(int i, int s) {
 // upper part U of the blocks.
 template <typename V>
 __global__ void block_y_kernel(const QDesc *__restrict__ qd, const double2 *const *__restrict__ VB,
-                               const V *__restrict__ Z, double2 *__restrict__ Y, long long RSc, int P, int N0) {
+                               const V *__restrict__ Z, double2 *__restrict__ Y, long long RSc, long long ldY, int P, int N0) {
     const QDesc q = qd[blockIdx.y];
     const double2 *vb = VB[blockIdx.y];
     long long total = q.ncols * N0;
@@ -213,7 +213,7 @@ __global__ void block_y_kernel(const QDesc *__restrict__ qd, const double2 *cons
             const double w = upper_weight(i, s);
             acc = cfma(make_double2(w * row[s].x, w * row[s].y), make_double2((double)zs.x, (double)zs.y), acc);
         }
-        Y[col * RSc + u] = acc;
+        Y[col * ldY + u] = acc;
     }
 }
 
@@ -244,7 +244,7 @@ __device__ __forceinline__ void split_f64(double x, float &hi, float &lo) {
 template <int P>
 __global__ void block_y_df_kernel(const QDesc *__restrict__ qd, const double2 *const *__restrict__ VB,
                                   const double2 *const *__restrict__ VD, const double2 *__restrict__ Z,
-                                  double2 *__restrict__ Y, long long RSc, int N0) {
+                                  double2 *__restrict__ Y, long long RSc, long long ldY, int N0) {
     extern __shared__ float4 vbs[];   // [N0 * P] blocks, then [N0] couplings: (hi re, lo re, hi im, lo im)
     const QDesc q = qd[blockIdx.y];
     const double2 *vb = VB[blockIdx.y];
@@ -294,7 +294,7 @@ __global__ void block_y_df_kernel(const QDesc *__restrict__ qd, const double2 *c
                 df_mac(v.x, v.y, zih[s], zil[s], Si, Ei);
                 df_mac(v.z, v.w, zrh[s], zrl[s], Si, Ei);
             }
-            Y[col * RSc + ch * (P - 1) + i] = make_double2(f32pair_to_f64(Sr, Er, 0), f32pair_to_f64(Si, Ei, 0));
+            Y[col * ldY + ch * (P - 1) + i] = make_double2(f32pair_to_f64(Sr, Er, 0), f32pair_to_f64(Si, Ei, 0));
         }
         if (VD) {
             // the channel's mu != 0 row: add its couplings to the mu = 0 functions
@@ -307,7 +307,7 @@ __global__ void block_y_df_kernel(const QDesc *__restrict__ qd, const double2 *c
                 df_mac(v.x, v.y, zih[s], zil[s], Si, Ei);
                 df_mac(v.z, v.w, zrh[s], zrl[s], Si, Ei);
             }
-            double2 *y = Y + col * RSc + N0 + ch;
+            double2 *y = Y + col * ldY + N0 + ch;
             const double2 y0 = *y;
             *y = make_double2(y0.x + f32pair_to_f64(Sr, Er, 0), y0.y + f32pair_to_f64(Si, Ei, 0));
         }
@@ -896,7 +896,7 @@ bool block_y_couples(int P, int N0) { return P >= 2 && P <= 4 && N0 > 0 && N0 % 
 
 template <typename V>
 void launch_block_y(const QDesc *d_q, int nq, const double2 *const *d_VB, const double2 *const *d_VD, const V *d_Z,
-                    double2 *d_Y, long long RSc, int P, int N0, long long maxcols, cudaStream_t st) {
+                    double2 *d_Y, long long RSc, long long ldY, int P, int N0, long long maxcols, cudaStream_t st) {
     if (N0 == 0 || nq == 0) return;
     long long per = maxcols * N0;
     long long g = (per + 255) / 256;
@@ -907,18 +907,18 @@ void launch_block_y(const QDesc *d_q, int nq, const double2 *const *d_VB, const 
             const long long per_df = maxcols * (N0 / (P - 1));
             const dim3 grid_df((unsigned)std::min<long long>(8192, (per_df + 255) / 256), (unsigned)nq);
             const size_t sm = (size_t)N0 * (P + 1) * sizeof(float4);
-            if (P == 2) block_y_df_kernel<2><<<grid_df, 256, sm, st>>>(d_q, d_VB, d_VD, d_Z, d_Y, RSc, N0);
-            else if (P == 3) block_y_df_kernel<3><<<grid_df, 256, sm, st>>>(d_q, d_VB, d_VD, d_Z, d_Y, RSc, N0);
-            else block_y_df_kernel<4><<<grid_df, 256, sm, st>>>(d_q, d_VB, d_VD, d_Z, d_Y, RSc, N0);
+            if (P == 2) block_y_df_kernel<2><<<grid_df, 256, sm, st>>>(d_q, d_VB, d_VD, d_Z, d_Y, RSc, ldY, N0);
+            else if (P == 3) block_y_df_kernel<3><<<grid_df, 256, sm, st>>>(d_q, d_VB, d_VD, d_Z, d_Y, RSc, ldY, N0);
+            else block_y_df_kernel<4><<<grid_df, 256, sm, st>>>(d_q, d_VB, d_VD, d_Z, d_Y, RSc, ldY, N0);
             return;
         }
     }
-    block_y_kernel<V><<<grid, 256, 0, st>>>(d_q, d_VB, d_Z, d_Y, RSc, P, N0);
+    block_y_kernel<V><<<grid, 256, 0, st>>>(d_q, d_VB, d_Z, d_Y, RSc, ldY, P, N0);
 }
 template void launch_block_y<float2>(const QDesc *, int, const double2 *const *, const double2 *const *, const float2 *,
-                                     double2 *, long long, int, int, long long, cudaStream_t);
+                                     double2 *, long long, long long, int, int, long long, cudaStream_t);
 template void launch_block_y<double2>(const QDesc *, int, const double2 *const *, const double2 *const *,
-                                      const double2 *, double2 *, long long, int, int, long long, cudaStream_t);
+                                      const double2 *, double2 *, long long, long long, int, int, long long, cudaStream_t);
 
 // Tiles of GEMM1 for one batch.  The A operand is the upper triangle U of the
 // dense block, so a row tile's K range (in each half) starts at its first row:
