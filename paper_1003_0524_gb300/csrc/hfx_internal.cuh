@@ -369,7 +369,8 @@ int launch_gemm2_tc(hfx_ctx *ctx, const __nv_bfloat16 *d_ZS, const __nv_bfloat16
 struct ZipwBuild {                          // per build: rows (k', m), segment grid, C slices
     bool ok = false;
     int R = 0, Rpad = 0, nmtile = 0, nL = 0, gx0 = 0, gy0 = 0, By = 0, nsegp_max = 0, Kp = 0;
-    int NBt = 0, nblk = 0, nbpad = 0, nzb = 0, nb_max = 0;
+    int NBt = 0, nblk = 0, nbpad = 0, nyb = 0, nzb = 0, nb_max = 0;
+    int ly = 0, lz = 2;                     // a segment is 2^ly y by 2^lz z values
     int tlo[3] = {0, 0, 0}, tdim[3] = {0, 0, 0};
     int sx0 = 0, sx1 = 0, sy0 = 0, sy1 = 0, sz0 = 0, sz1 = 0;   // extent of the segment starts
     std::vector<int> rowbase;               // first row of every k'

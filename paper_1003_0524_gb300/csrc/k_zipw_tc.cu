@@ -5,19 +5,23 @@
 // For a fixed k and a fixed shift W = G - G0, every (k', m) row of every pair
 // (k, q) that needs this W is one row of a GEMM
 //   Z[(k', m), n] = sum_{G1} C[(k', m), G1] T_k[n](W + G1),   C = conj(c),
-// whose reduction index G1 runs over the plane waves of all k' in segments of
-// 4 consecutive z values along the (x, y) lines of the plane-wave spheres.
+// whose reduction index G1 runs over the plane waves of all k' in segments of 4
+// points: 4 consecutive z values along the (x, y) lines of the plane-wave spheres, or
+// patches of 2 y by 2 z values, whichever covers the spheres with fewer segments (the
+// rest of a segment is padding).  2 atoms, 485 plane waves: 720 points as lines, 660 as
+// patches, uneven band counts 55.4 ms against 58.1 in the interstitial kernel; 10 atoms, 297: 408 and 400; 5 atoms, 179: 304
+// and 308, lines.
 //
 // Operands (fixed-point slices of tc_ptx.cuh, real embedding of the complex
 // product with the real and imaginary outputs side by side in N); one segment
-// is 8 K values, the real and imaginary parts of its 4 z values:
-//   A row (k', m) = [ Re C(4 z) | Im C(4 z) ] per segment   (128-byte swizzle, 2-D TMA)
-//   B rows        = [ T_r(4 z) | -T_i(4 z) ] (real out), [ T_i(4 z) | T_r(4 z) ] (imag out)
-// The sliced T box is stored in blocks of 4 z with all planes and both output
+// is 8 K values, the real and imaginary parts of its 4 points:
+//   A row (k', m) = [ Re C(4) | Im C(4) ] per segment   (128-byte swizzle, 2-D TMA)
+//   B rows        = [ T_r(4) | -T_i(4) ] (real out), [ T_i(4) | T_r(4) ] (imag out)
+// The sliced T box is stored in blocks of one segment with all planes and both output
 // rows of all bands of a band block contiguous, so the B operand of one
 // segment is a single 1-D bulk copy (no swizzle).  A copy must start on a
-// 16-byte boundary, i.e. at a multiple of 4 in z: T is kept in four copies
-// shifted by 0, 1, 2, 3 in z, so a segment may start at any z.
+// 16-byte boundary, i.e. at a block: T is kept in four copies shifted by every
+// (y, z) inside a block, so a segment may start anywhere.
 #include <algorithm>
 #include <memory>
 #include <string>
@@ -32,10 +36,12 @@ using namespace tc;
 namespace {
 
 constexpr int ZT_BM = 128;
-// K chunk: KSEG segments of 8 K values.  Band blocks up to 40 take 8 segments
-// (64 K, 128-byte swizzle, two stages); larger ones 4 (32 K, 64-byte swizzle,
-// three stages), so that the stages of a 64-band tile still fit
-__host__ __device__ constexpr int zt_kseg(int NB) { return NB > 40 ? 4 : 8; }
+// K chunk: KSEG segments of 8 K values.  Band blocks up to 48 take 8 segments
+// (64 K, 128-byte swizzle, two stages: half the waits and commits per K); larger ones 4
+// (32 K, 64-byte swizzle, three stages), since two stages of a 64-band tile with 8 do not
+// fit the 227 KB.  Interstitial kernel with 4 and 8 segments: 2 atoms, 40 bands, 32.5 and
+// 31.9 ms; 48 bands, uneven, 55.4 and 54.2; blocks of 8 bands 115.6 and 88.0.
+__host__ __device__ constexpr int zt_kseg(int NB) { return NB > 48 ? 4 : 8; }
 __host__ __device__ constexpr int zt_stages(int KSEG) { return KSEG == 8 ? 2 : 3; }
 constexpr int ZT_EPI = 8;
 constexpr int ZT_THREADS = 128 + 32 * ZT_EPI;   // warpgroup 0: producer, MMA (2 idle); 1, 2: epilogue
@@ -45,8 +51,9 @@ constexpr int ZT_THREADS = 128 + 32 * ZT_EPI;   // warpgroup 0: producer, MMA (2
 __host__ __device__ constexpr bool zt_split(int NB) { return NB >= 56; }
 constexpr int ZT_REG_LAUNCH = 168, ZT_REG_CTRL = 64, ZT_REG_EPI = 216;
 static_assert(4 * ZT_REG_CTRL + 8 * ZT_REG_EPI <= 12 * ZT_REG_LAUNCH, "register split exceeds the launch allocation");
-constexpr int ZT_SEGZ = 4;                 // z values per segment (8 K values: real and imaginary parts)
-constexpr int ZT_NCOPY = ZT_SEGZ;          // z-shifted copies of the sliced T box
+constexpr int ZT_PTS = 4;                  // points per segment (8 K values: real and imaginary parts)
+constexpr int ZT_NCOPY = ZT_PTS;           // shifted copies of the sliced T box
+// a segment is 2^ly y by 2^lz z values, ly + lz = 2
 
 __device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
     return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
@@ -55,13 +62,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 lo, __nv_bfloat16 
 // ------------------------------------------------------------- C slices
 // One block per row r = (k', m) of c scaled by Omega^{-1/2}: exponent over
 // |Re c|, |Im c| of the row, then
-// Re C = c_r at K = 8 s + j and Im C = -c_i at K = 8 s + 4 + j, where segment
-// s = segstart + (z - z0) / 4 and j = (z - z0) mod 4 on the segment grid of the
-// row's tile.
+// Re C = c_r at K = 8 s + j and Im C = -c_i at K = 8 s + 4 + j, where segment s and
+// point j of a plane wave follow from the segment grid of the row's tile: per line the
+// first segment and the line's y inside it (segstart = 2 s + dy), and the first z.
 __global__ void c_slices_kernel(const double2 *const *__restrict__ ck, const int *const *__restrict__ Gk,
                                 const int *__restrict__ npw_k, const int *__restrict__ rowk, const int *__restrict__ rowm,
                                 const int *__restrict__ line_of, int gx0, int gy0, int By, int nL,
-                                const int *__restrict__ segstart, const int *__restrict__ segz0, int Kp, int Rpad,
+                                const int *__restrict__ segstart, const int *__restrict__ segz0, int lz, int Kp, int Rpad,
                                 double rs, __nv_bfloat16 *__restrict__ A, int *__restrict__ aexp) {
     int r = blockIdx.x;
     int kp = rowk[r], m = rowm[r];
@@ -87,13 +94,13 @@ __global__ void c_slices_kernel(const double2 *const *__restrict__ ck, const int
         slice4(rs * c[i].x, e, sr);
         slice4(-(rs * c[i].y), e, si);
         const size_t sl = (size_t)(r / ZT_BM) * nL + li;   // segment grid of the row's tile
-        const int dz = z - segz0[sl];
-        const long long K = (long long)(segstart[sl] + dz / ZT_SEGZ) * 8 + dz % ZT_SEGZ;
+        const int dz = z - segz0[sl], ss = segstart[sl];
+        const long long K = (long long)((ss >> 1) + (dz >> lz)) * 8 + ((ss & 1) << lz) + (dz & ((1 << lz) - 1));
 #pragma unroll
         for (int p = 0; p < NPL; ++p) {
             __nv_bfloat16 *row = A + ((long long)p * Rpad + r) * Kp;
             row[K] = sr[p];
-            row[K + ZT_SEGZ] = si[p];
+            row[K + ZT_PTS] = si[p];
         }
     }
 }
@@ -118,39 +125,41 @@ __global__ void t_exp_kernel(const double2 *const *__restrict__ Tk, const int *_
     if (threadIdx.x == 0) eT[(size_t)k * nbmax + n] = line_exp_bits(red[0]);
 }
 
-// Slices of T: one thread per (k, cell (X, Y, zb), band n) slices the 7 values
-// T_k[n](X, Y, 4 zb .. 4 zb + 6) once and writes, for every copy c (T shifted
-// by c in z) and plane p, the two B rows of band n = b NB + j over the 4 z
-// values 4 zb + c .. 4 zb + c + 3:
-//   Tq[c][k][X][Y][zb][b][p][j]      = [ Re T (4 z) | -Im T (4 z) ]   (real output)
-//   Tq[c][k][X][Y][zb][b][p][NB + j] = [ Im T (4 z) |  Re T (4 z) ]   (imaginary output)
-// (16 bytes each); bands past nb(k) and z past the box are 0.  Consecutive
+// Slices of T: one thread per (k, cell (X, yb, zb), band n) slices the values of T_k[n]
+// around its cell once (7 z for lines, 3 x 3 for patches) and writes, for every copy c
+// (T shifted inside a block) and plane p, the two B rows of band n = b NB + j over the 4
+// points of the block:
+//   Tq[c][k][X][yb][zb][b][p][j]      = [ Re T (4) | -Im T (4) ]   (real output)
+//   Tq[c][k][X][yb][zb][b][p][NB + j] = [ Im T (4) |  Re T (4) ]   (imaginary output)
+// (16 bytes each); bands past nb(k) and points past the box are 0.  Consecutive
 // threads take consecutive bands, so the row stores are coalesced.  One
-// (c, k, X, Y, zb, b) block -- all planes of one segment -- is contiguous.
+// (c, k, X, yb, zb, b) block -- all planes of one segment -- is contiguous.
+template <int LY>
 __global__ void t_slices_kernel(const double2 *const *__restrict__ Tk, const int *__restrict__ nb_k, int td0, int td1,
-                                int td2, int nzb, int NB, int nblk, int nbmax, int nslot, const int *__restrict__ kslot,
-                                const int *__restrict__ eT, __nv_bfloat16 *__restrict__ Tq) {
-    constexpr int NZ = ZT_SEGZ + ZT_NCOPY - 1;                // z values a thread needs
+                                int td2, int nyb, int nzb, int NB, int nblk, int nbmax, int nslot,
+                                const int *__restrict__ kslot, const int *__restrict__ eT, __nv_bfloat16 *__restrict__ Tq) {
+    constexpr int LZ = 2 - LY, SY = 1 << LY, SZ = 1 << LZ;
+    constexpr int NY = 2 * SY - 1, NZ = 2 * SZ - 1;           // values a thread needs
     const int k = blockIdx.y;
     const int slot = kslot[k];
     if (slot < 0) return;
     const int nbpad = NB * nblk;
-    const long long ncell = (long long)td0 * td1 * nzb;
+    const long long ncell = (long long)td0 * nyb * nzb;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ncell * nbpad) return;
     const int n = (int)(idx % nbpad);
-    const long long cellk = idx / nbpad;                      // (X, Y, zb) of this k
+    const long long cellk = idx / nbpad;                      // (X, yb, zb) of this k
     const int zb = (int)(cellk % nzb);
-    const long long xy = cellk / nzb;
+    const int yb = (int)((cellk / nzb) % nyb), X = (int)(cellk / ((long long)nzb * nyb));
     const bool live = n < nb_k[k];
     const long long box = (long long)td0 * td1 * td2;
-    const double2 *T = live ? Tk[k] + (size_t)n * box + xy * td2 : nullptr;
+    const double2 *T = live ? Tk[k] + (size_t)n * box + (size_t)X * td1 * td2 : nullptr;
     const int e = live ? eT[(size_t)k * nbmax + n] : 0;
-    __nv_bfloat16 sr[NZ][NPL], si[NZ][NPL];
+    __nv_bfloat16 sr[NY * NZ][NPL], si[NY * NZ][NPL];
 #pragma unroll
-    for (int t = 0; t < NZ; ++t) {
-        const int z = zb * ZT_SEGZ + t;
-        const double2 v = (live && z < td2) ? T[z] : make_double2(0.0, 0.0);
+    for (int t = 0; t < NY * NZ; ++t) {
+        const int y = yb * SY + t / NZ, z = zb * SZ + t % NZ;
+        const double2 v = (live && y < td1 && z < td2) ? T[(size_t)y * td2 + z] : make_double2(0.0, 0.0);
         slice4(v.x, e, sr[t]);
         slice4(v.y, e, si[t]);
     }
@@ -160,15 +169,19 @@ __global__ void t_slices_kernel(const double2 *const *__restrict__ Tk, const int
     for (int c = 0; c < ZT_NCOPY; ++c) {
         const long long cell = ((long long)c * nslot + slot) * ncell + cellk;
         __nv_bfloat16 *dst = Tq + (cell * nblk + b) * (NPL * blk) + (long long)j * 8;
+        // copy c: shifted by (c >> LZ, c mod SZ); its points (i >> LZ, i mod SZ)
+        int at[ZT_PTS];
+#pragma unroll
+        for (int i = 0; i < ZT_PTS; ++i) at[i] = ((c >> LZ) + (i >> LZ)) * NZ + (c & (SZ - 1)) + (i & (SZ - 1));
 #pragma unroll
         for (int p = 0; p < NPL; ++p) {
             uint4 ro, io;   // real-output row, imaginary-output row
-            ro.x = pack_bf16x2(sr[c][p], sr[c + 1][p]);
-            ro.y = pack_bf16x2(sr[c + 2][p], sr[c + 3][p]);
-            ro.z = pack_bf16x2(__hneg(si[c][p]), __hneg(si[c + 1][p]));
-            ro.w = pack_bf16x2(__hneg(si[c + 2][p]), __hneg(si[c + 3][p]));
-            io.x = pack_bf16x2(si[c][p], si[c + 1][p]);
-            io.y = pack_bf16x2(si[c + 2][p], si[c + 3][p]);
+            ro.x = pack_bf16x2(sr[at[0]][p], sr[at[1]][p]);
+            ro.y = pack_bf16x2(sr[at[2]][p], sr[at[3]][p]);
+            ro.z = pack_bf16x2(__hneg(si[at[0]][p]), __hneg(si[at[1]][p]));
+            ro.w = pack_bf16x2(__hneg(si[at[2]][p]), __hneg(si[at[3]][p]));
+            io.x = pack_bf16x2(si[at[0]][p], si[at[1]][p]);
+            io.y = pack_bf16x2(si[at[2]][p], si[at[3]][p]);
             io.z = ro.x;
             io.w = ro.y;
             *reinterpret_cast<uint4 *>(dst + p * blk) = ro;
@@ -193,12 +206,12 @@ struct ZParams {
     const int *rowk, *rowm;       // rows of A (k', m)
     const int *aexp, *eT;         // row exponents, [k][n] band exponents
     const int *kslot;             // k -> slot of its T slices
-    const int2 *segoff;           // [row tile][segment] (x td1 + y of its line, z0)
+    const int2 *segoff;           // [row tile][segment] (x | y << 16 of its first line, z0)
     int nsegp_max;
     const int *nchunk;            // [row tile] 64-K chunks
     const int *runs;              // [row tile][chunk] bit j: segment j of the chunk starts a bulk copy; bits 8..: live segments
     const __nv_bfloat16 *Tq;      // sliced T blocks (t_slices_kernel layout)
-    int td0, td1, nzb, nblk, nslot;
+    int td0, nyb, nzb, ly, lz, nblk, nslot;
     double2 *ZI;                  // output plane ZI[g][col] (rows g of the interstitial part, G-major)
     long long NCi;                // row stride of ZI: the columns of the batch
     int nmt, nk, R, Rpad, nbmax, tlo0, tlo1, tlo2;
@@ -273,11 +286,10 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
             const int slot = p.kslot[tl.k];
             const int2 *so = p.segoff + (size_t)gt * p.nsegp_max;
             const int *runs = p.runs + (size_t)gt * (p.nsegp_max / KSEG);
-            // a segment starts at X = W_x + x - tlo_x, Y likewise, and T z index
-            // Zs = W_z - tlo_z + z0: copy Zs mod 4, z block Zs / 4 -- inside the
-            // box by construction
-            const int bxy = (W.x - p.tlo0) * p.td1 + (W.y - p.tlo1);
-            const int bz = W.z - p.tlo2;
+            // a segment starts at X = W_x + x - tlo_x, Ys and Zs likewise: the copy
+            // follows from Ys and Zs modulo the block, the block from the quotients --
+            // inside the box by construction
+            const int bx = W.x - p.tlo0, by = W.y - p.tlo1, bz = W.z - p.tlo2;
             bool stop = false;
             int ri_next = nch > 0 ? runs[0] : 0;
             int2 sg_next = (nch > 0 && lane < KSEG) ? so[lane] : make_int2(0, 0);
@@ -301,10 +313,10 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
                 if (lane < live && ((starts >> lane) & 1)) {
                     const int rest = starts >> (lane + 1);
                     const int len = rest ? __ffs(rest) : live - lane;   // segments up to the next run
-                    const int Zs = bz + sg.y;
-                    const int cp = Zs & (ZT_NCOPY - 1);
+                    const int X = bx + (int)(short)sg.x, Ys = by + (sg.x >> 16), Zs = bz + sg.y;
+                    const int cp = ((Ys & ((1 << p.ly) - 1)) << p.lz) | (Zs & ((1 << p.lz) - 1));
                     const long long cell =
-                        (((long long)cp * p.nslot + slot) * ((long long)p.td0 * p.td1) + bxy + sg.x) * p.nzb + Zs / ZT_SEGZ;
+                        ((((long long)cp * p.nslot + slot) * p.td0 + X) * p.nyb + (Ys >> p.ly)) * p.nzb + (Zs >> p.lz);
                     bulk_load(saddr(st + NPL * ZT_A_PLANE + lane * SEG4), tq + (cell * p.nblk + tl.nblk) * SEG4,
                               (uint32_t)(len * SEG4), &full_bar[s]);
                 }
@@ -588,10 +600,20 @@ int zipw_tc_plan_build(hfx_ctx *ctx, const std::vector<int> &kset, int nb_max, c
     std::vector<std::vector<int>> tile_k(nmtile);
     for (int r = 0; r < R; ++r)
         if (tile_k[r / ZT_BM].empty() || tile_k[r / ZT_BM].back() != rowk[r]) tile_k[r / ZT_BM].push_back(rowk[r]);
-    // segment grid per row tile: the lines of the tile's spheres, each cut
-    // into segments of ZT_SEGZ z values from its lowest z
-    std::vector<int> segstart((size_t)nmtile * nL, 0), segz0((size_t)nmtile * nL, 0), nseg(nmtile);
-    std::vector<std::vector<int4>> segs(nmtile);
+    // segment grid per row tile: the lines of the tile's spheres, each (or each pair of
+    // neighbours in y) cut into segments from its lowest z; both kinds are laid out and
+    // the one with fewer segments is taken
+    struct Grid {
+        std::vector<int> start, z0;              // [tile][line] 2 segment + y inside it, first z
+        std::vector<std::vector<int4>> segs;     // [tile] (x, y, z) of every segment
+        long long total = 0;
+    } grids[2];
+    for (auto &g : grids) {
+        g.start.assign((size_t)nmtile * nL, 0);
+        g.z0.assign((size_t)nmtile * nL, 0);
+        g.segs.resize(nmtile);
+    }
+    std::vector<int> nseg(nmtile);
     std::vector<int> tzlo(nL), tzhi(nL);
     for (int t = 0; t < nmtile; ++t) {
         std::fill(tzlo.begin(), tzlo.end(), 1 << 29);
@@ -604,19 +626,56 @@ int zipw_tc_plan_build(hfx_ctx *ctx, const std::vector<int> &kset, int nb_max, c
                 tzhi[l] = std::max(tzhi[l], G[i + 2]);
             }
         }
-        for (int l = 0; l < nL; ++l) {
-            if (tzlo[l] > tzhi[l]) continue;
-            segstart[(size_t)t * nL + l] = (int)segs[t].size();
-            segz0[(size_t)t * nL + l] = tzlo[l];
-            for (int z = tzlo[l]; z <= tzhi[l]; z += ZT_SEGZ) segs[t].push_back(make_int4(lx[l], ly[l], z, 0));
+        // lines l, l2 (l2 < 0: one line) as segments of 2^lz z values
+        auto put = [&](Grid &g, int l, int l2, int lz) {
+            const int z0 = l2 < 0 ? tzlo[l] : std::min(tzlo[l], tzlo[l2]), z1 = l2 < 0 ? tzhi[l] : std::max(tzhi[l], tzhi[l2]);
+            const int s = (int)g.segs[t].size();
+            g.start[(size_t)t * nL + l] = 2 * s;
+            g.z0[(size_t)t * nL + l] = z0;
+            if (l2 >= 0) {
+                g.start[(size_t)t * nL + l2] = 2 * s + 1;
+                g.z0[(size_t)t * nL + l2] = z0;
+            }
+            for (int z = z0; z <= z1; z += 1 << lz) g.segs[t].push_back(make_int4(lx[l], ly[l], z, 0));
+        };
+        auto live = [&](int l) { return l < nL && tzlo[l] <= tzhi[l]; };
+        for (int l = 0; l < nL; ++l)
+            if (live(l)) put(grids[0], l, -1, 2);
+        for (int l0 = 0; l0 < nL;) {             // lines of one x, ascending y
+            int l1 = l0;
+            while (l1 < nL && lx[l1] == lx[l0]) ++l1;
+            // pairs (y, y + 1) from the first line on, or that line alone first: fewer segments
+            auto walk = [&](bool alone, bool lay) {
+                int n = 0;
+                for (int l = l0; l < l1;) {
+                    if (!live(l)) { ++l; continue; }
+                    const bool pair = !alone && l + 1 < l1 && live(l + 1) && ly[l + 1] == ly[l] + 1;
+                    const int z0 = pair ? std::min(tzlo[l], tzlo[l + 1]) : tzlo[l], z1 = pair ? std::max(tzhi[l], tzhi[l + 1]) : tzhi[l];
+                    n += (z1 - z0) / 2 + 1;
+                    if (lay) put(grids[1], l, pair ? l + 1 : -1, 1);
+                    l += pair ? 2 : 1;
+                    alone = false;
+                }
+                return n;
+            };
+            const bool alone = walk(true, false) < walk(false, false);
+            walk(alone, true);
+            l0 = l1;
         }
-        if (segs[t].empty()) segs[t].push_back(make_int4(lx[0], ly[0], lzlo[0], 0));
-        nseg[t] = (int)segs[t].size();
+        for (Grid &g : grids) {
+            if (g.segs[t].empty()) g.segs[t].push_back(make_int4(lx[0], ly[0], lzlo[0], 0));
+            g.total += (long long)g.segs[t].size();
+        }
     }
+    zb.ly = grids[1].total < grids[0].total ? 1 : 0;
+    zb.lz = 2 - zb.ly;
+    const std::vector<int> &segstart = grids[zb.ly].start, &segz0 = grids[zb.ly].z0;
+    const std::vector<std::vector<int4>> &segs = grids[zb.ly].segs;
+    for (int t = 0; t < nmtile; ++t) nseg[t] = (int)segs[t].size();
     int nsegp_max = 0;
     for (int t = 0; t < nmtile; ++t) nsegp_max = std::max(nsegp_max, (nseg[t] + 7) / 8 * 8);
     const int Kp = nsegp_max * 8;   // K values of an A row: 8 per segment
-    const int nzb = (tdim[2] + ZT_SEGZ - 1) / ZT_SEGZ;
+    const int nyb = (tdim[1] + (1 << zb.ly) - 1) >> zb.ly, nzb = (tdim[2] + (1 << zb.lz) - 1) >> zb.lz;
     const int NBt = zipw_tc_valid_nb(nb_tile) ? nb_tile : pick_nb(nb_max);
     const int nblk = (nb_max + NBt - 1) / NBt;
     const int KSEG = zt_kseg(NBt);   // segments per K chunk of the kernel instance
@@ -626,11 +685,11 @@ int zipw_tc_plan_build(hfx_ctx *ctx, const std::vector<int> &kset, int nb_max, c
         nchunk[t] = (nseg[t] + KSEG - 1) / KSEG;
         for (int s2 = 0; s2 < nsegp_max; ++s2) {
             const int4 sg = s2 < nseg[t] ? segs[t][s2] : segs[t][0];   // padding: any valid block
-            segtab[(size_t)t * nsegp_max + s2] = make_int2(sg.x * tdim[1] + sg.y, sg.z);
+            segtab[(size_t)t * nsegp_max + s2] = make_int2((int)((unsigned)(unsigned short)(short)sg.x | (unsigned)sg.y << 16), sg.z);
         }
     }
     // bulk-copy runs per K chunk: consecutive segments of one line are
-    // consecutive z blocks of T, contiguous for a single band block
+    // consecutive z blocks of T (same copy), contiguous for a single band block
     std::vector<int> runs((size_t)nmtile * (nsegp_max / KSEG), 0);
     for (int t = 0; t < nmtile; ++t)
         for (int c = 0; c < nsegp_max / KSEG; ++c) {
@@ -639,7 +698,7 @@ int zipw_tc_plan_build(hfx_ctx *ctx, const std::vector<int> &kset, int nb_max, c
             for (int j = 0; j < live; ++j) {
                 const int s2 = KSEG * c + j;
                 const bool cont = j > 0 && nblk == 1 && segs[t][s2].x == segs[t][s2 - 1].x &&
-                                  segs[t][s2].y == segs[t][s2 - 1].y && segs[t][s2].z == segs[t][s2 - 1].z + ZT_SEGZ;
+                                  segs[t][s2].y == segs[t][s2 - 1].y && segs[t][s2].z == segs[t][s2 - 1].z + (1 << zb.lz);
                 if (!cont) starts |= 1 << j;
             }
             runs[(size_t)t * (nsegp_max / KSEG) + c] = starts | (live << 8);
@@ -672,10 +731,10 @@ int zipw_tc_plan_build(hfx_ctx *ctx, const std::vector<int> &kset, int nb_max, c
     zb.s_eT = lay.place((size_t)nk * nb_max * 4);
     zb.scratch_bytes = lay.off;
     zb.R = R; zb.Rpad = Rpad; zb.nmtile = nmtile; zb.nL = nL; zb.gx0 = gmin[0]; zb.gy0 = gmin[1]; zb.By = By;
-    zb.nsegp_max = nsegp_max; zb.Kp = Kp; zb.NBt = NBt; zb.nblk = nblk; zb.nbpad = nblk * NBt; zb.nzb = nzb;
+    zb.nsegp_max = nsegp_max; zb.Kp = Kp; zb.NBt = NBt; zb.nblk = nblk; zb.nbpad = nblk * NBt; zb.nyb = nyb; zb.nzb = nzb;
     zb.nb_max = nb_max;
     for (int x = 0; x < 3; ++x) { zb.tlo[x] = tlo[x]; zb.tdim[x] = tdim[x]; }
-    zb.tq_bytes_per_slot = (size_t)ZT_NCOPY * tdim[0] * tdim[1] * nzb * NPL * 2 * zb.nbpad * 8 * 2;
+    zb.tq_bytes_per_slot = (size_t)ZT_NCOPY * tdim[0] * nyb * nzb * NPL * 2 * zb.nbpad * 8 * 2;
     zb.ok = true;
     return HFX_OK;
 }
@@ -751,7 +810,7 @@ int zipw_tc_plan_batch(hfx_ctx *ctx, const ZipwBuild &zb, const std::vector<int>
     for (const int4 &W : wxyz) {
         const int Z0 = W.z + zb.sz0 - zb.tlo[2], Z1 = W.z + zb.sz1 - zb.tlo[2];
         if (W.x + zb.sx0 - zb.tlo[0] < 0 || W.x + zb.sx1 - zb.tlo[0] >= zb.tdim[0] || W.y + zb.sy0 - zb.tlo[1] < 0 ||
-            W.y + zb.sy1 - zb.tlo[1] >= zb.tdim[1] || Z0 < 0 || Z1 / ZT_SEGZ >= zb.nzb)
+            W.y + zb.sy1 - zb.tlo[1] >= zb.tdim[1] || Z0 < 0 || Z1 >= zb.tdim[2])
             return set_err(ctx, HFX_EUNSUPPORTED, "interstitial segment outside the step-function box");
     }
     if (tiles.size() > (size_t)0x7fffffff) return set_err(ctx, HFX_EUNSUPPORTED, "interstitial tile list too long");
@@ -781,7 +840,7 @@ int zipw_tc_run_build(hfx_ctx *ctx, const ZipwBuild &zb, const char *dtab, char 
                                           reinterpret_cast<const int *>(dtab + zb.o_rowm),
                                           reinterpret_cast<const int *>(dtab + zb.o_line), zb.gx0, zb.gy0, zb.By, zb.nL,
                                           reinterpret_cast<const int *>(dtab + zb.o_sst),
-                                          reinterpret_cast<const int *>(dtab + zb.o_sz0), zb.Kp, zb.Rpad,
+                                          reinterpret_cast<const int *>(dtab + zb.o_sz0), zb.lz, zb.Kp, zb.Rpad,
                                           1.0 / sqrt(ctx->omega), A, aexp);
     t_exp_kernel<<<dim3(zb.nb_max, ctx->nk), 256, 0, st>>>(d_Tk, d_nb, zb.tdim[0], zb.tdim[1], zb.tdim[2], zb.nb_max,
                                                            reinterpret_cast<const int *>(dtab + zb.o_kall), eT);
@@ -800,9 +859,10 @@ int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, co
     int rc;
     const int *kslot = reinterpret_cast<const int *>(dtab + bt.o_kslot);
     {
-        const long long nthreads = (long long)zb.tdim[0] * zb.tdim[1] * zb.nzb * zb.nbpad;
-        t_slices_kernel<<<dim3((unsigned)((nthreads + 255) / 256), ctx->nk), 256, 0, st>>>(
-            d_Tk, d_nb, zb.tdim[0], zb.tdim[1], zb.tdim[2], zb.nzb, zb.NBt, zb.nblk, zb.nb_max, bt.nslot, kslot,
+        const long long nthreads = (long long)zb.tdim[0] * zb.nyb * zb.nzb * zb.nbpad;
+        auto kern = zb.ly ? t_slices_kernel<1> : t_slices_kernel<0>;
+        kern<<<dim3((unsigned)((nthreads + 255) / 256), ctx->nk), 256, 0, st>>>(
+            d_Tk, d_nb, zb.tdim[0], zb.tdim[1], zb.tdim[2], zb.nyb, zb.nzb, zb.NBt, zb.nblk, zb.nb_max, bt.nslot, kslot,
             reinterpret_cast<const int *>(dscr + zb.s_eT), dTq);
     }
     if ((rc = cuda_check(ctx, cudaGetLastError(), "zipw T slices"))) return rc;
@@ -829,8 +889,10 @@ int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, co
     p.runs = reinterpret_cast<const int *>(dtab + zb.o_runs);
     p.Tq = dTq;
     p.td0 = zb.tdim[0];
-    p.td1 = zb.tdim[1];
+    p.nyb = zb.nyb;
     p.nzb = zb.nzb;
+    p.ly = zb.ly;
+    p.lz = zb.lz;
     p.nblk = zb.nblk;
     p.nslot = bt.nslot;
     p.ZI = d_ZI;
