@@ -311,7 +311,7 @@ template <typename V>
 void launch_slice_cols(const V *d_Z, long long RSc, const QDesc *d_q, int nq, long long NC, long long maxcols, int N0,
                        int N0pad, int HS, int RS, __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st);
 // The slices of Z with the interstitial rows still in the G-major plane ZI [g][NCi].
-int launch_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long NCi, const double2 *d_Z, long long RSc, const QDesc *d_q,
+int launch_slice_z(hfx_ctx *ctx, const float4 *d_ZI, long long NCi, const int *d_cexp, const double2 *d_Z, long long RSc, const QDesc *d_q,
                    int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
                    __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st);
 // The channel blocks of Y' = U Z (rows [0, N0)), U the upper triangle of v_t
@@ -346,7 +346,8 @@ ModSizes apply_mod_sizes(int maxD);
 int apply_mod_prepare_u(hfx_ctx *ctx, const double2 *d_VD, __nv_bfloat16 *d_UR, int *d_uexp, int D, int naux, int N0,
                         const ModSizes &z);
 int apply_mod_tiles(const QDesc *h_q, int nq, std::vector<unsigned char> &out);
-int apply_mod_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long sg, long long sc, const double2 *d_Z, long long RSc,
+// d_ZI null: the interstitial rows are in Z
+int apply_mod_slice_z(hfx_ctx *ctx, const float4 *d_ZI, const int *d_cexp, const double2 *d_Z, long long RSc,
                       const QDesc *d_q, int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
                       const ModSizes &z, __nv_bfloat16 *d_ZS, __nv_bfloat16 *d_ZR, int *d_xexp, int *d_zexp);
 int apply_mod_run(hfx_ctx *ctx, const __nv_bfloat16 *d_UR_all, int nk, const __nv_bfloat16 *d_ZR, short *d_YR, long long NC,
@@ -374,7 +375,7 @@ struct ZipwBuild {                          // per build: rows (k', m), segment 
     int tlo[3] = {0, 0, 0}, tdim[3] = {0, 0, 0};
     int sx0 = 0, sx1 = 0, sy0 = 0, sy1 = 0, sz0 = 0, sz1 = 0;   // extent of the segment starts
     std::vector<int> rowbase;               // first row of every k'
-    size_t o_rowk = 0, o_rowm = 0, o_line = 0, o_sst = 0, o_sz0 = 0, o_seg = 0, o_nch = 0, o_runs = 0, o_kall = 0;
+    size_t o_rowk = 0, o_rowm = 0, o_rb = 0, o_line = 0, o_sst = 0, o_sz0 = 0, o_seg = 0, o_nch = 0, o_runs = 0, o_kall = 0;
     size_t s_a = 0, s_aexp = 0, s_eT = 0, scratch_bytes = 0, a_elems = 0;
     size_t tq_bytes_per_slot = 0;           // sliced T of one k (all copies, planes, bands)
 };
@@ -393,10 +394,11 @@ int zipw_tc_plan_batch(hfx_ctx *ctx, const ZipwBuild &zb, const std::vector<int>
 int zipw_tc_run_build(hfx_ctx *ctx, const ZipwBuild &zb, const char *dtab, char *dscr, const double2 *const *d_ck,
                       const int *const *d_Gk, const int *d_npw, const double2 *const *d_Tk, const int *d_nb);
 // The interstitial rows come out G-major into d_ZI [g][NCi] (the kernel's stores then
-// fill whole sectors); with transpose they are also put into d_Z after the kernel.
+// fill whole sectors) as FP32 pairs in units of 2^d_cexp[col]; with transpose they are
+// also put into d_Z, in FP64, after the kernel.
 int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, const char *dtab, const char *dscr,
                       __nv_bfloat16 *dTq, const PairDesc *d_pairs, const double2 *const *d_Tk, const int *d_nb,
-                      double2 *d_Z, long long RSc, double2 *d_ZI, long long NCi, const QDesc *d_qd, int nq,
+                      int npairs, double2 *d_Z, long long RSc, float4 *d_ZI, long long NCi, int *d_cexp, const QDesc *d_qd, int nq,
                       long long maxcols, int max_nipw, bool transpose, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch);
 
 // ------------------------------------------------------------ stage-1 products on the tensor cores (k_cgemm_tc.cu)

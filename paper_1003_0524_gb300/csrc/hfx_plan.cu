@@ -410,7 +410,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         size_t praw = tc ? (size_t)((hnb[ik] + NB - 1) / NB) * ((hnb[ik] + NB - 1) / NB) * (2 * NB) * (2 * NB) * sizeof(double)
                          : (size_t)ksplit * hnb[ik] * hnb[ik] * sizeof(double2);
         size_t b = (size_t)nc * z_bytes + praw + nc * y_bytes;
-        if (tc) b += nc * ((size_t)4 * pl.RS * sizeof(__nv_bfloat16) + ys_bytes + 3 * sizeof(int));
+        if (tc) b += nc * ((size_t)4 * pl.RS * sizeof(__nv_bfloat16) + ys_bytes + 4 * sizeof(int));
         if (pl.mod) b += (size_t)nc * N0 * sizeof(double2);
         return b;
     };
@@ -536,7 +536,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         pl.zipw_tq_off = zl.place(std::max<size_t>(max_tq, 256));
         if ((rc = scratch_reserve(ctx, ctx->s_zs, (size_t)4 * ncol_max * pl.RS * sizeof(__nv_bfloat16))) ||
             (rc = scratch_reserve(ctx, ctx->s_ys, ncol_max * ys_bytes)) ||
-            (rc = scratch_reserve(ctx, ctx->s_xexp, (size_t)3 * ncol_max * sizeof(int))) ||
+            (rc = scratch_reserve(ctx, ctx->s_xexp, (size_t)4 * ncol_max * sizeof(int))) ||
             (rc = scratch_reserve(ctx, ctx->s_cgT, std::max<size_t>(pl.tp.scratch_bytes, 256))) ||
             (rc = scratch_reserve(ctx, ctx->s_cgZ, std::max<size_t>(pl.zmt.scratch_bytes, 256))) ||
             (rc = scratch_reserve(ctx, ctx->s_zipw, zl.off)))
@@ -741,8 +741,10 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
         }
         rec(ctx, bt.ev[1]);
         // the slicing kernel reads the interstitial rows where the interstitial kernel
-        // left them; only a caller's projections or keep_products need them in Z
+        // left them (also with keep_products, so that the result is the same); Z gets them
+        // for keep_products and, to be sliced there, beside a caller's projections
         const bool z_whole = keep || !bt.overrides.empty();
+        int *cexp = tc ? reinterpret_cast<int *>(ctx->s_xexp.p) + 3 * bt.ncols : nullptr;   // exponents of the plane's columns
         int max_nipw = 0;
         for (auto &q : bt.qd) max_nipw = std::max(max_nipw, q.nipw);
         if (tc && sizeof(R) == 8) {
@@ -751,8 +753,8 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             if ((rc = zipw_tc_run_batch(ctx, pl.zipw, bt.zipw, tab, reinterpret_cast<char *>(ctx->s_zipw.p),
                                         at<__nv_bfloat16>(ctx->s_zipw.p, pl.zipw_tq_off), d_pairs,
                                         reinterpret_cast<const double2 *const *>(tab + pl.o_T),
-                                        reinterpret_cast<const int *>(tab + pl.o_nb), reinterpret_cast<double2 *>(Zc), RSc,
-                                        Yd, bt.ncols, d_qd, nq, bt.maxcols, max_nipw, z_whole,
+                                        reinterpret_cast<const int *>(tab + pl.o_nb), npairs, reinterpret_cast<double2 *>(Zc), RSc,
+                                        reinterpret_cast<float4 *>(Yd), bt.ncols, cexp, d_qd, nq, bt.maxcols, max_nipw, z_whole,
                                         bt.ev[2], bt.ev[3], &nl)))
                 return rc;
         } else {
@@ -802,20 +804,20 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             int *zexp = reinterpret_cast<int *>(ctx->s_xexp.p), *yexp = zexp + bt.ncols;
             int *mexp = yexp + bt.ncols;   // powers of two of the residues of Z
             // the interstitial rows: in the interstitial kernel's plane, or in Z
-            const bool in_z = z_whole || !bt.zipw.ok;
+            const bool in_z = !bt.overrides.empty() || !bt.zipw.ok;
             double2 *Y0 = reinterpret_cast<double2 *>(ctx->s_pairs.p);   // modular apply: mu = 0 rows of Y'
             if (pl.mod) {
                 // (before the apply, which takes the place of Z)
                 launch_block_y<V>(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb), nullptr, Zc, Y0, RSc, N0,
                                   P, N0, bt.maxcols, ctx->stream);
                 const double2 *Zd = reinterpret_cast<const double2 *>(Zc);
-                if ((rc = apply_mod_slice_z(ctx, in_z ? Zd + nmt : Yd, in_z ? 1 : bt.ncols, in_z ? RSc : 1, Zd, RSc, d_qd, nq,
+                if ((rc = apply_mod_slice_z(ctx, in_z ? nullptr : reinterpret_cast<const float4 *>(Yd), cexp, Zd, RSc, d_qd, nq,
                                             bt.ncols, bt.maxcols, nmt, N0, pl.N0pad, pl.HS, pl.RS, pl.ms, ZS, YS, zexp, mexp)))
                     return rc;
             } else if (in_z) {
                 launch_slice_cols<V>(Zc, RSc, d_qd, nq, bt.ncols, bt.maxcols, N0, pl.N0pad, pl.HS, pl.RS, ZS, zexp, ctx->stream);
                 if ((rc = cuda_check(ctx, cudaGetLastError(), "slice kernels"))) return rc;
-            } else if ((rc = launch_slice_z(ctx, Yd, bt.ncols, reinterpret_cast<double2 *>(Zc), RSc, d_qd, nq, bt.ncols,
+            } else if ((rc = launch_slice_z(ctx, reinterpret_cast<const float4 *>(Yd), bt.ncols, cexp, reinterpret_cast<double2 *>(Zc), RSc, d_qd, nq, bt.ncols,
                                             bt.maxcols, nmt, N0, pl.N0pad, pl.HS, pl.RS, ZS, zexp, ctx->stream))) {
                 return rc;
             }

@@ -112,6 +112,13 @@ __device__ __forceinline__ uint64_t f2_both(float x) { return f2_pack(__float_as
 
 // round(|x| 2^s) with the sign of x, for |x| 2^s < 2^36 (0 for zeros and subnormals),
 // as three 12-bit pieces x = p2 2^24 + p1 2^12 + p0, |p0|, |p1| <= 2048, |p2| <= 2107
+__device__ __forceinline__ void pieces_of(long long N, float (&p)[3]) {
+    const unsigned long long v = (unsigned long long)N + 0x800800800ULL;
+    const uint32_t vl = (uint32_t)v, vh = (uint32_t)(v >> 32);
+    p[0] = __uint_as_float(0x4B000000u | (vl & 0xfffu)) - 8390656.0f;
+    p[1] = __uint_as_float(0x4B000000u | ((vl >> 12) & 0xfffu)) - 8390656.0f;
+    p[2] = __int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 24)) - 12584960.0f;
+}
 __device__ __forceinline__ void int_pieces(double x, int s, float (&p)[3]) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
     const int E = (int)((hi >> 20) & 0x7ffu);
@@ -119,11 +126,7 @@ __device__ __forceinline__ void int_pieces(double x, int s, float (&p)[3]) {
     const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
     const unsigned long long q = ((sh < 64 ? m >> sh : 0ULL) + 1) >> 1;
     const unsigned long long neg = (unsigned long long)((long long)(int)hi >> 63);
-    const unsigned long long v = (q ^ neg) - neg + 0x800800800ULL;
-    const uint32_t vl = (uint32_t)v, vh = (uint32_t)(v >> 32);
-    p[0] = __uint_as_float(0x4B000000u | (vl & 0xfffu)) - 8390656.0f;
-    p[1] = __uint_as_float(0x4B000000u | ((vl >> 12) & 0xfffu)) - 8390656.0f;
-    p[2] = __int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 24)) - 12584960.0f;
+    pieces_of((long long)((q ^ neg) - neg), p);
 }
 
 // p - m round(p / m) for packed integers |p| < 2^22
@@ -238,13 +241,15 @@ __global__ void __launch_bounds__(256) mod_u_kernel(const double2 *__restrict__ 
 
 // ------------------------------------------------------------- Z
 // The digits of Z (all rows, for Z^H Y) and the residues of its dense rows (for the
-// apply), from the interstitial rows ZI [g sg + col sc] (the plane of the interstitial
-// kernel, or Z itself where a caller's projections are in it) and the muffin-tin rows of
-// Z; the layout and the passes of slice_z_kernel, with the sum of squares of the dense rows
-// beside the maximum.  Bound by memory: 32 bytes read, 48 written per element.
+// apply), from the interstitial rows (F32: the interstitial kernel's plane ZI [g][col] of
+// FP32 pairs in units of 2^cexp[col]; else Z itself, where a caller's projections are in
+// it) and the muffin-tin rows of Z; the layout and the passes of slice_z_kernel, with the
+// sum of squares of the dense rows beside the maximum.  Bound by memory: 32 bytes read, 48 written per element.
 constexpr int MZ_COLS = 8, MZ_THREADS = 256, MZ_NJ = MZ_THREADS / MZ_COLS, MZ_CH = 4 * MZ_NJ, MZ_CS = MZ_CH + 8;
 constexpr size_t kMzSmem = (size_t)(2 * NPL + NC16) * MZ_COLS * MZ_CS * sizeof(__nv_bfloat16);
-__global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const double2 *__restrict__ ZI, long long sg, long long sc,
+template <bool F32>
+__global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const float4 *__restrict__ ZI, long long NCi,
+                                                           const int *__restrict__ cexp,
                                                            const double2 *__restrict__ Z, long long RSc,
                                                            const QDesc *__restrict__ qd, int nmt, int N0, int N0pad, int HS,
                                                            int RS, int Kp, long long NC, __nv_bfloat16 *__restrict__ XS,
@@ -262,19 +267,29 @@ __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const double2 *__r
     const int tid = threadIdx.x, c = tid % MZ_COLS, j = tid / MZ_COLS;
     const bool live = c0 + c < q.ncols;
     const long long col = q.colbase + (live ? c0 + c : c0);
-    const double2 *z = Z + col * RSc, *zi = ZI + col * sc;
+    const double2 *z = Z + col * RSc;
+    const float4 *zi = ZI + col;
+    const int ce = F32 ? cexp[col] : 0;
     unsigned long long mx = 0;
     SquareSum n;
-    for (int i = j; i < nmt; i += NJ) {
+    for (int i = j; i < (F32 ? nmt : nmt + q.nipw); i += NJ) {
         const double2 v = z[i];
         mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
         if (i >= N0) n.add(v);
     }
-#pragma unroll 4
-    for (int g = j; g < q.nipw; g += NJ) {
-        const double2 v = zi[(size_t)g * sg];
-        mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
-        n.add(v);
+    if (F32) {
+        // sums of integers below 2^30 in units of the column's exponent: no scale needed
+        uint32_t mf = 0;
+        float s = 0.0f;
+#pragma unroll 8
+        for (int g = j; g < q.nipw; g += NJ) {
+            const float4 v = zi[(size_t)g * NCi];
+            mf = max(mf, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.z) & 0x7fffffffu));
+            s = fmaf(v.x, v.x, fmaf(v.z, v.z, s));
+        }
+        const unsigned long long mp = abs_bits(f32pair_to_f64_int(__uint_as_float(mf), 0.0f, ce));   // 0 below the normal range
+        mx = max(mx, mp);
+        if (mp) n.join(1023 + ce + 16, s * 0x1p-32f);
     }
 #pragma unroll
     for (int o = 8; o <= 16; o <<= 1) {
@@ -292,18 +307,18 @@ __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const double2 *__r
     if (j == 0 && live) { xexp[col] = e; zexp[col] = sb; }
     const int nd = nmt - N0;                       // muffin-tin rows among the dense ones
     const long long plane = NC * RS, rplane = NC * Kp;
-    double2 v[4];                                  // this thread's four rows of a chunk
+    uint4 v[4];                                    // this thread's four rows of a chunk, as they are
     auto fetch = [&](int u) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const int dr = u + t - N0pad;          // dense row
-            v[t] = make_double2(0.0, 0.0);
-            if (dr >= nd) {
-                if (dr < q.D) v[t] = zi[(size_t)(dr - nd) * sg];
+            v[t] = make_uint4(0, 0, 0, 0);
+            if (F32 && dr >= nd) {
+                if (dr < q.D) v[t] = *reinterpret_cast<const uint4 *>(zi + (size_t)(dr - nd) * NCi);
             } else if (dr >= 0) {
-                v[t] = z[N0 + dr];
+                if (dr < q.D) v[t] = *reinterpret_cast<const uint4 *>(z + N0 + dr);
             } else if (u + t < N0) {
-                v[t] = z[u + t];
+                v[t] = *reinterpret_cast<const uint4 *>(z + u + t);
             }
         }
     };
@@ -314,10 +329,7 @@ __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const double2 *__r
         {
             Digits sr[4], si[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                sr[t] = slice4f(v[t].x, e);
-                si[t] = slice4f(v[t].y, e);
-            }
+            for (int t = 0; t < 4; ++t) slice_row(v[t], F32 && u0 + 4 * j + t - N0pad >= nd, e, ce, sr[t], si[t]);
 #pragma unroll
             for (int p = 0; p < NPL; ++p) {
                 __nv_bfloat16 *s = stage + (size_t)((2 * p) * MZ_COLS + c) * CS + 4 * j;
@@ -330,8 +342,13 @@ __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const double2 *__r
             float x[4][3], y[4][3];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                int_pieces(v[t].x, sb, x[t]);
-                int_pieces(v[t].y, sb, y[t]);
+                if (F32 && u0 + 4 * j + t - N0pad >= nd) {
+                    pieces_of(pair_round<20>(__uint_as_float(v[t].x), __uint_as_float(v[t].y), sb + ce), x[t]);
+                    pieces_of(pair_round<20>(__uint_as_float(v[t].z), __uint_as_float(v[t].w), sb + ce), y[t]);
+                } else {
+                    int_pieces(__hiloint2double((int)v[t].y, (int)v[t].x), sb, x[t]);
+                    int_pieces(__hiloint2double((int)v[t].w, (int)v[t].z), sb, y[t]);
+                }
             }
             uint64_t X[2][3], Y[2][3];
 #pragma unroll
@@ -813,14 +830,18 @@ int apply_mod_tiles(const QDesc *h_q, int nq, std::vector<unsigned char> &out) {
     return (int)tiles.size();
 }
 
-int apply_mod_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long sg, long long sc, const double2 *d_Z, long long RSc, const QDesc *d_q,
-                      int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS, const ModSizes &z,
-                      __nv_bfloat16 *d_ZS, __nv_bfloat16 *d_ZR, int *d_xexp, int *d_zexp) {
+int apply_mod_slice_z(hfx_ctx *ctx, const float4 *d_ZI, const int *d_cexp, const double2 *d_Z, long long RSc,
+                      const QDesc *d_q, int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
+                      const ModSizes &z, __nv_bfloat16 *d_ZS, __nv_bfloat16 *d_ZR, int *d_xexp, int *d_zexp) {
     if (nq == 0 || maxcols == 0) return HFX_OK;
-    cudaFuncSetAttribute(mod_z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMzSmem);
     const dim3 grid((unsigned)((maxcols + MZ_COLS - 1) / MZ_COLS), (unsigned)nq);
-    mod_z_kernel<<<grid, MZ_THREADS, kMzSmem, ctx->stream>>>(d_ZI, sg, sc, d_Z, RSc, d_q, nmt, N0, N0pad, HS, RS, z.Kp, NC, d_ZS,
-                                                             d_ZR, d_xexp, d_zexp);
+    auto go = [&](auto kern) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMzSmem);
+        kern<<<grid, MZ_THREADS, kMzSmem, ctx->stream>>>(d_ZI, NC, d_cexp, d_Z, RSc, d_q, nmt, N0, N0pad, HS, RS, z.Kp, NC, d_ZS,
+                                                         d_ZR, d_xexp, d_zexp);
+    };
+    if (d_ZI) go(mod_z_kernel<true>);
+    else go(mod_z_kernel<false>);
     return cuda_check(ctx, cudaGetLastError(), "residues of Z");
 }
 

@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(256, 4) slice_cols_kernel(const V *__restrict_
 }
 
 // The same slices of the projections Z, whose interstitial rows come from the G-major
-// plane ZI [g][col] of the interstitial kernel and whose muffin-tin rows from Z: the
+// plane ZI [g][col] of the interstitial kernel (FP32 pairs in units of 2^cexp[col]) and
+// whose muffin-tin rows from Z: the
 // transposition, the column maximum and the slicing in one kernel.  A block takes
 // SZ_COLS = 8 adjacent columns (128 bytes of every ZI row); it reads them twice and
 // turns chunks of 128 rows around in shared memory, so that the planes are written in
@@ -106,8 +107,8 @@ __global__ void __launch_bounds__(256, 4) slice_cols_kernel(const V *__restrict_
 // the two reads leaves too few warps (9.4 ms), as does bounding the columns in flight
 // so that the second read hits L2 (7.6 ms); 16 columns or 128 threads change nothing.
 constexpr int SZ_COLS = 8, SZ_THREADS = 256;
-__global__ void __launch_bounds__(SZ_THREADS) slice_z_kernel(const double2 *__restrict__ ZI, long long NCi,
-                                                          const double2 *__restrict__ Z, long long RSc,
+__global__ void __launch_bounds__(SZ_THREADS) slice_z_kernel(const float4 *__restrict__ ZI, long long NCi,
+                                                          const int *__restrict__ cexp, const double2 *__restrict__ Z, long long RSc,
                                                           const QDesc *__restrict__ qd, int nmt, int N0, int N0pad, int HS,
                                                           int RS, long long NC, __nv_bfloat16 *__restrict__ XS,
                                                           int *__restrict__ xexp) {
@@ -120,17 +121,22 @@ __global__ void __launch_bounds__(SZ_THREADS) slice_z_kernel(const double2 *__re
     const int tid = threadIdx.x, c = tid % SZ_COLS, j = tid / SZ_COLS;
     const bool live = c0 + c < q.ncols;
     const long long col = q.colbase + (live ? c0 + c : c0);
-    const double2 *z = Z + col * RSc, *zi = ZI + col;
+    const double2 *z = Z + col * RSc;
+    const float4 *zi = ZI + col;
+    const int ce = cexp[col];
+    // the maximum as the bits of a double (muffin-tin rows) and of a float (plane), made one
     unsigned long long mx = 0;
+    uint32_t mf = 0;
     for (int i = j; i < nmt; i += NJ) {
         const double2 v = z[i];
         mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
     }
 #pragma unroll 8
     for (int g = j; g < q.nipw; g += NJ) {
-        const double2 v = zi[(size_t)g * NCi];
-        mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
+        const float4 v = zi[(size_t)g * NCi];
+        mf = max(mf, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.z) & 0x7fffffffu));
     }
+    mx = max(mx, abs_bits(f32pair_to_f64_int(__uint_as_float(mf), 0.0f, ce)));
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
     if (tid % 32 < SZ_COLS) red[tid / 32][c] = mx;
@@ -141,18 +147,18 @@ __global__ void __launch_bounds__(SZ_THREADS) slice_z_kernel(const double2 *__re
     if (j == 0 && live) xexp[col] = e;
     const int nd = nmt - N0;                       // muffin-tin rows among the dense ones
     const long long plane = NC * RS;
-    double2 v[4];                                  // this thread's four rows of a chunk
+    uint4 v[4];                                    // this thread's four rows of a chunk, as they are
     auto fetch = [&](int u) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const int dr = u + t - N0pad;          // dense row
-            v[t] = make_double2(0.0, 0.0);
+            v[t] = make_uint4(0, 0, 0, 0);
             if (dr >= nd) {
-                if (dr < q.D) v[t] = zi[(size_t)(dr - nd) * NCi];
+                if (dr < q.D) v[t] = *reinterpret_cast<const uint4 *>(zi + (size_t)(dr - nd) * NCi);
             } else if (dr >= 0) {
-                v[t] = z[N0 + dr];
+                v[t] = *reinterpret_cast<const uint4 *>(z + N0 + dr);
             } else if (u + t < N0) {
-                v[t] = z[u + t];
+                v[t] = *reinterpret_cast<const uint4 *>(z + u + t);
             }
         }
     };
@@ -160,10 +166,7 @@ __global__ void __launch_bounds__(SZ_THREADS) slice_z_kernel(const double2 *__re
     for (int u0 = 0; u0 < HS; u0 += CH) {
         Digits sr[4], si[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            sr[t] = slice4f(v[t].x, e);
-            si[t] = slice4f(v[t].y, e);
-        }
+        for (int t = 0; t < 4; ++t) slice_row(v[t], u0 + 4 * j + t - N0pad >= nd, e, ce, sr[t], si[t]);
         if (u0 + CH < HS) fetch(u0 + CH + 4 * j);  // the next chunk, while this one is stored
         __syncthreads();                           // the chunk before has been stored
 #pragma unroll
@@ -883,12 +886,12 @@ template void launch_slice_cols<float2>(const float2 *, long long, const QDesc *
 template void launch_slice_cols<double2>(const double2 *, long long, const QDesc *, int, long long, long long, int, int,
                                          int, int, __nv_bfloat16 *, int *, cudaStream_t);
 
-int launch_slice_z(hfx_ctx *ctx, const double2 *d_ZI, long long NCi, const double2 *d_Z, long long RSc, const QDesc *d_q,
+int launch_slice_z(hfx_ctx *ctx, const float4 *d_ZI, long long NCi, const int *d_cexp, const double2 *d_Z, long long RSc, const QDesc *d_q,
                    int nq, long long NC, long long maxcols, int nmt, int N0, int N0pad, int HS, int RS,
                    __nv_bfloat16 *d_XS, int *d_exp, cudaStream_t st) {
     if (nq == 0 || maxcols == 0) return HFX_OK;
     const dim3 grid((unsigned)((maxcols + SZ_COLS - 1) / SZ_COLS), (unsigned)nq);
-    slice_z_kernel<<<grid, SZ_THREADS, 0, st>>>(d_ZI, NCi, d_Z, RSc, d_q, nmt, N0, N0pad, HS, RS, NC, d_XS, d_exp);
+    slice_z_kernel<<<grid, SZ_THREADS, 0, st>>>(d_ZI, NCi, d_cexp, d_Z, RSc, d_q, nmt, N0, N0pad, HS, RS, NC, d_XS, d_exp);
     return cuda_check(ctx, cudaGetLastError(), "slice kernel");
 }
 

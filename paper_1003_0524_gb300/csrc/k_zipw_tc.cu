@@ -204,7 +204,6 @@ struct ZParams {
     const int *gtab;              // [nq][ax][ay][az] aux index or -1
     int ax0, ay0, az0, ad0, ad1, ad2;
     const int *rowk, *rowm;       // rows of A (k', m)
-    const int *aexp, *eT;         // row exponents, [k][n] band exponents
     const int *kslot;             // k -> slot of its T slices
     const int2 *segoff;           // [row tile][segment] (x | y << 16 of its first line, z0)
     int nsegp_max;
@@ -212,7 +211,7 @@ struct ZParams {
     const int *runs;              // [row tile][chunk] bit j: segment j of the chunk starts a bulk copy; bits 8..: live segments
     const __nv_bfloat16 *Tq;      // sliced T blocks (t_slices_kernel layout)
     int td0, nyb, nzb, ly, lz, nblk, nslot;
-    double2 *ZI;                  // output plane ZI[g][col] (rows g of the interstitial part, G-major)
+    float4 *ZI;                   // output plane ZI[g][col] (rows g of the interstitial part, G-major)
     long long NCi;                // row stride of ZI: the columns of the batch
     int nmt, nk, R, Rpad, nbmax, tlo0, tlo1, tlo2;
     double rs;                    // Omega^{-1/2}
@@ -238,7 +237,6 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
     __shared__ uint64_t full_bar[ZT_STAGES], empty_bar[ZT_STAGES], tfull_bar, tempty_bar, mma_done;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
-    __shared__ int s_eT[ZT_EPI][32];      // per epilogue warp: the band exponents of its bands
     int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     // B segments of every stage start as zeros: padding segments are never loaded
     for (int s = 0; s < ZT_STAGES; ++s) {
@@ -401,17 +399,11 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
             const int ngroups = (p.nchunk[tl.mrow / ZT_BM] + ZT_GROUP - 1) / ZT_GROUP;   // same grouping as the MMA warp
             // everything the output of this row needs, fetched now so that the
             // dependent loads overlap the first K group instead of following it:
-            // the output row g, the first column and the live bands, the scales
-            int g = -1, nlive = 0, ea = 0;
+            // the output row g, the first column and the live bands
+            int g = -1, nlive = 0;
             long long col = 0;
             {
-                // the band exponents of this warp's bands (the same for every row of
-                // the tile: one k) go to shared memory, one per lane; the row's own
-                // exponent stays in a register
                 const int n0 = tl.nblk * NB + cs * NH;
-                __syncwarp();
-                s_eT[e][lane] = (lane < NH && n0 + lane < p.nbmax) ? p.eT[(size_t)tl.k * p.nbmax + n0 + lane] : 0;
-                __syncwarp();
                 const int r = tl.mrow + quarter * 32 + lane;
                 if (r < p.R) {
                     const int kp = p.rowk[r], m = p.rowm[r];
@@ -423,7 +415,6 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
                             g = p.gtab[(((size_t)pr.qslot * p.ad0 + Gx) * p.ad1 + Gy) * p.ad2 + Gz];
                         nlive = min(NH, pr.nb - n0);
                         col = pr.col0 + (long long)m * pr.nb + n0;
-                        ea = p.aexp[r] - 16;
                     }
                 }
             }
@@ -464,21 +455,25 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
             if (!ok) break;
             if (g >= 0) {
                 // G-major: this row's bands are consecutive columns of row g, so the
-                // thread's stores fill whole sectors (the transpose into Z follows)
-                double2 *out = p.ZI + (size_t)g * p.NCi + col;
+                // thread's stores fill whole sectors.  A value leaves as the FP32 pair
+                // (s, e), s + e = hi + lo exactly and s its rounding, in units of the
+                // column's exponent (col_exp_kernel): what reads the plane cuts the digits
+                // from the pair.  Turning it into FP64 here, 90 integer instructions per
+                // element while the single accumulator waits, left the tensor cores idle for
+                // 0.29 of the kernel's time at 40 bands.  Interstitial kernel 31.7 to
+                // 26.1 ms (40 bands), 54.1 to 45.5 (uneven), 6.4 to 4.8 (10 atoms).
+                float4 *out = p.ZI + (size_t)g * p.NCi + col;
+                const bool al = ((uintptr_t)out & 31) == 0;
 #pragma unroll
-                for (int jj = 0; jj < NH; ++jj) {
-                    if (jj < nlive) {
-                        const float2 h1 = f2_unpack(hr[jj / 2]), l1 = f2_unpack(lr[jj / 2]);
-                        const float2 h2 = f2_unpack(hm[jj / 2]), l2 = f2_unpack(lm[jj / 2]);
-                        const bool odd = jj & 1;
-                        // Omega^{-1/2} is in the C slices; the conversion runs on the integer
-                        // units (measured faster here than the one-FP64-add form)
-                        double2 v;
-                        const int ex = ea + s_eT[e][jj];
-                        v.x = f32pair_to_f64_int(odd ? h1.y : h1.x, odd ? l1.y : l1.x, ex);
-                        v.y = f32pair_to_f64_int(odd ? h2.y : h2.x, odd ? l2.y : l2.x, ex);
-                        __stcs(out + jj, v);   // streaming: keep the operands in L2
+                for (int jj = 0; jj < NH; jj += 2) {
+                    float2 sr, er, si, ei;
+                    f2_two_sum(hr[jj / 2], lr[jj / 2], sr, er);
+                    f2_two_sum(hm[jj / 2], lm[jj / 2], si, ei);
+                    if (al && jj + 1 < nlive) {
+                        st_global_32(out + jj, make_float4(sr.x, er.x, si.x, ei.x), make_float4(sr.y, er.y, si.y, ei.y));
+                    } else {
+                        if (jj < nlive) __stcs(out + jj, make_float4(sr.x, er.x, si.x, ei.x));
+                        if (jj + 1 < nlive) __stcs(out + jj + 1, make_float4(sr.y, er.y, si.y, ei.y));
                     }
                 }
             }
@@ -492,13 +487,22 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zipw_tc_kernel(const __grid_con
     }
 }
 
+// The exponent of every column of the plane ZI: that of its row (k', m) of C plus that of
+// band n of T (one block per pair).
+__global__ void col_exp_kernel(const PairDesc *__restrict__ pairs, const int *__restrict__ rowbase,
+                               const int *__restrict__ aexp, const int *__restrict__ eT, int nbmax, int *__restrict__ cexp) {
+    const PairDesc pr = pairs[blockIdx.x];
+    for (int i = threadIdx.x; i < pr.no * pr.nb; i += blockDim.x)
+        cexp[pr.col0 + i] = aexp[rowbase[pr.ikp] + i / pr.nb] - 16 + eT[(size_t)pr.ik * nbmax + i % pr.nb];
+}
+
 // Z[col][nmt + g] = ZI[g][col] for the interstitial rows g < nipw(q) of every
-// column of every q of the batch: 32 x 32 tiles through shared memory, reads
-// along the columns of ZI and writes along the rows of Z, both coalesced.
-__global__ void __launch_bounds__(256) ipw_transpose_kernel(const double2 *__restrict__ ZI, long long NCi,
-                                                            double2 *__restrict__ Z, long long RSc, int nmt,
-                                                            const QDesc *__restrict__ qd) {
-    __shared__ double2 tile[32][33];
+// column of every q of the batch, as FP64 numbers: 32 x 32 tiles through shared memory,
+// reads along the columns of ZI and writes along the rows of Z, both coalesced.
+__global__ void __launch_bounds__(256) ipw_transpose_kernel(const float4 *__restrict__ ZI, long long NCi,
+                                                            const int *__restrict__ cexp, double2 *__restrict__ Z,
+                                                            long long RSc, int nmt, const QDesc *__restrict__ qd) {
+    __shared__ float4 tile[32][33];
     const QDesc q = qd[blockIdx.z];
     const long long c0 = (long long)blockIdx.x * 32;
     const int g0 = blockIdx.y * 32;
@@ -515,7 +519,12 @@ __global__ void __launch_bounds__(256) ipw_transpose_kernel(const double2 *__res
     for (int i = 0; i < 4; ++i) {
         const long long c = c0 + ty + 8 * i;
         const int g = g0 + tx;
-        if (g < q.nipw && c < q.ncols) Z[(size_t)(q.colbase + c) * RSc + nmt + g] = tile[tx][ty + 8 * i];
+        if (g < q.nipw && c < q.ncols) {
+            const float4 f = tile[tx][ty + 8 * i];
+            const int e = cexp[q.colbase + c];
+            Z[(size_t)(q.colbase + c) * RSc + nmt + g] =
+                make_double2(f32pair_to_f64_int(f.x, f.y, e), f32pair_to_f64_int(f.z, f.w, e));
+        }
     }
 }
 
@@ -716,6 +725,7 @@ int zipw_tc_plan_build(hfx_ctx *ctx, const std::vector<int> &kset, int nb_max, c
     for (int ik : kset) kall[ik] = 0;
     zb.o_rowk = tab.put(rowk);
     zb.o_rowm = tab.put(rowm);
+    zb.o_rb = tab.put(zb.rowbase);
     zb.o_line = tab.put(line_of);
     zb.o_sst = tab.put(segstart);
     zb.o_sz0 = tab.put(segz0);
@@ -852,8 +862,8 @@ int zipw_tc_valid_nb(int nb) { return nb >= 8 && nb <= 64 && nb % 8 == 0; }
 // Per batch: T slices of the batch's k and the GEMM.
 int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, const char *dtab, const char *dscr,
                       __nv_bfloat16 *dTq, const PairDesc *d_pairs, const double2 *const *d_Tk, const int *d_nb,
-                      double2 *d_Z, long long RSc, double2 *d_ZI, long long NCi, const QDesc *d_qd, int nq,
-                      long long maxcols, int max_nipw, bool transpose, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch) {
+                      int npairs, double2 *d_Z, long long RSc, float4 *d_ZI, long long NCi, int *d_cexp, const QDesc *d_qd,
+                      int nq, long long maxcols, int max_nipw, bool transpose, cudaEvent_t ev0, cudaEvent_t ev1, int *nlaunch) {
     if (!zb.ok || !bt.ok) return HFX_OK;
     cudaStream_t st = ctx->stream;
     int rc;
@@ -880,8 +890,6 @@ int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, co
     p.ad0 = bt.ad[0]; p.ad1 = bt.ad[1]; p.ad2 = bt.ad[2];
     p.rowk = reinterpret_cast<const int *>(dtab + zb.o_rowk);
     p.rowm = reinterpret_cast<const int *>(dtab + zb.o_rowm);
-    p.aexp = reinterpret_cast<const int *>(dscr + zb.s_aexp);
-    p.eT = reinterpret_cast<const int *>(dscr + zb.s_eT);
     p.kslot = kslot;
     p.segoff = reinterpret_cast<const int2 *>(dtab + zb.o_seg);
     p.nsegp_max = zb.nsegp_max;
@@ -939,11 +947,14 @@ int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, co
     }
     if (rc_launch) return rc_launch;
     if ((rc = cuda_check(ctx, cudaGetLastError(), "zipw tensor-core kernel"))) return rc;
+    col_exp_kernel<<<(unsigned)npairs, 256, 0, st>>>(d_pairs, reinterpret_cast<const int *>(dtab + zb.o_rb),
+                                                     reinterpret_cast<const int *>(dscr + zb.s_aexp),
+                                                     reinterpret_cast<const int *>(dscr + zb.s_eT), zb.nb_max, d_cexp);
     if (transpose && nq > 0 && maxcols > 0 && max_nipw > 0) {
         const dim3 tg((unsigned)((maxcols + 31) / 32), (unsigned)((max_nipw + 31) / 32), (unsigned)nq);
-        ipw_transpose_kernel<<<tg, 256, 0, st>>>(d_ZI, NCi, d_Z, RSc, ctx->nmt, d_qd);
+        ipw_transpose_kernel<<<tg, 256, 0, st>>>(d_ZI, NCi, d_cexp, d_Z, RSc, ctx->nmt, d_qd);
     }
-    if (nlaunch) *nlaunch += transpose ? 3 : 2;
+    if (nlaunch) *nlaunch += transpose ? 4 : 3;
     return cuda_check(ctx, cudaGetLastError(), "interstitial transpose");
 }
 

@@ -318,6 +318,30 @@ __device__ __forceinline__ Digits slice4f(double x, int e) {
     d.s[3] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.0f);
     return d;
 }
+// the digits of N, |N| <= 2^32
+__device__ __forceinline__ Digits digits_of(long long N) {
+    const unsigned long long v = (unsigned long long)N + 0x808080ULL;
+    const uint32_t vl = (uint32_t)v, vh = (uint32_t)(v >> 32);
+    Digits d;
+    d.s[0] = __float_as_uint(__int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 24)) - 12582912.0f);
+    d.s[1] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7442)) - 8388736.0f);
+    d.s[2] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7441)) - 8388736.0f);
+    d.s[3] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.0f);
+    return d;
+}
+// x 2^p as an integer with F fraction bits, truncated (|x| 2^(p + F) < 2^62)
+__device__ __forceinline__ long long f32_fixed(float x, int k) {   // k = p + F
+    const uint32_t b = __float_as_uint(x);
+    const int E = (int)((b >> 23) & 0xffu), sh = E - 150 + k;
+    const unsigned long long m = E ? (unsigned long long)((b & 0x7fffffu) | 0x800000u) : 0ULL;
+    const unsigned long long a = sh >= 0 ? m << min(sh, 39) : (sh > -24 ? m >> -sh : 0ULL);
+    return (int)b < 0 ? -(long long)a : (long long)a;
+}
+// round((s + e) 2^p), to nearest even as far as 2^-F of a unit
+template <int F> __device__ __forceinline__ long long pair_round(float s, float e, int p) {
+    const long long V = f32_fixed(s, p + F) + f32_fixed(e, p + F);
+    return (V + ((1LL << (F - 1)) - 1) + ((V >> F) & 1)) >> F;
+}
 // the BF16 patterns of two digits (their FP32 bits) in one word
 __device__ __forceinline__ uint32_t pack_digits(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
 
@@ -373,6 +397,20 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
     uint64_t r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+
+// s + e = h + l exactly, s = fl(h + l), for two columns at once
+__device__ __forceinline__ void f2_two_sum(uint64_t h, uint64_t l, float2 &s, float2 &e) {
+    const uint64_t t = f2_add(h, l), bb = f2_sub(t, h);
+    s = f2_unpack(t);
+    e = f2_unpack(f2_add(f2_sub(h, f2_sub(t, bb)), f2_sub(l, bb)));
+}
+// 32 bytes to global memory (32-byte aligned) in one store, not kept in L2
+__device__ __forceinline__ void st_global_32(void *p, const float4 &a, const float4 &b) {
+    asm volatile("st.global.cs.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(__float_as_uint(a.x)),
+                 "r"(__float_as_uint(a.y)), "r"(__float_as_uint(a.z)), "r"(__float_as_uint(a.w)), "r"(__float_as_uint(b.x)),
+                 "r"(__float_as_uint(b.y)), "r"(__float_as_uint(b.z)), "r"(__float_as_uint(b.w))
+                 : "memory");
 }
 
 // class_accumulate (sc = 1) for two columns at once; a_w hold the class sums
@@ -452,6 +490,18 @@ __device__ __forceinline__ double f32pair_to_f64_int(float h, float l, int k) {
     const long long bexp = (long long)(e0 + k - lz) + 63 + 1023;        // biased exponent of the leading bit
     if (bexp < 1) return 0.0;
     return __longlong_as_double((long long)(sgn | (((unsigned long long)(bexp - 1) << 52) + m)));
+}
+
+// The digits of one complex row of a column with exponent e: an FP64 pair, or an FP32
+// pair (s_r, e_r, s_i, e_i) in units of 2^ce.
+__device__ __forceinline__ void slice_row(const uint4 &v, bool f32, int e, int ce, Digits &re, Digits &im) {
+    if (f32) {
+        re = digits_of(pair_round<24>(__uint_as_float(v.x), __uint_as_float(v.y), 32 - e + ce));
+        im = digits_of(pair_round<24>(__uint_as_float(v.z), __uint_as_float(v.w), 32 - e + ce));
+    } else {
+        re = slice4f(__hiloint2double((int)v.y, (int)v.x), e);
+        im = slice4f(__hiloint2double((int)v.w, (int)v.z), e);
+    }
 }
 
 // S + E += a * b for double-FP32 a = (ah, al), b = (bh, bl): the product's
