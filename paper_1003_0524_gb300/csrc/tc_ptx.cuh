@@ -427,6 +427,11 @@ __device__ __forceinline__ void class_accumulate2(uint64_t a0, uint64_t a1, uint
     lo = f2_add(lo, f2_fma(c, s8, er));
 }
 
+// the bits of ldexpf(1, k), also where it is subnormal, zero or infinite
+__device__ __forceinline__ uint32_t pow2_bits(int k) {
+    return k >= -126 ? (uint32_t)(min(k, 128) + 127) << 23 : (k >= -149 ? 1u << (k + 149) : 0u);
+}
+
 // class_accumulate for two columns with per-column scales sc (packed pair)
 __device__ __forceinline__ void class_accumulate2_sc(uint64_t a0, uint64_t a1, uint64_t a2, uint64_t a3, uint64_t sc,
                                                      uint64_t &hi, uint64_t &lo) {
