@@ -61,6 +61,15 @@ def _profiled_traffic(kernel_file: str, profile: str):
     return int(m.group(1))
 
 
+def _apply_kernel(s, st):
+    """The kernel of the dense-block Coulomb apply and its tensor products per real
+    multiply-add: 10 digit products, or, for complex dense blocks of 1280 to 6144 rows,
+    4 residue products (16 for a complex one: 8 moduli, 2 real products each)."""
+    n_lm = s.n_atoms * (s.Lmax + 1) ** 2
+    D = max((n_lm if st["sparse_used"] else s.n_mt) + int(g.shape[0]) for g in s.Gaux)
+    return ("mod_gemm_kernel", 4.0) if not s.inversion and 1280 <= D <= 6144 else ("gemm1_kernel", 10.0)
+
+
 def _peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -412,26 +421,29 @@ def run_ours(args):
             "zipw": (avg("ms_zipw"), st["flops_zipw"]),
         }
         dom = max(kernels, key=lambda k: kernels[k][0])
-        names = {"apply": "gemm1_kernel", "zhy": "gemm2_kernel", "zipw": "zipw_tc_kernel"}
+        apply_name, apply_products = _apply_kernel(s, st)
+        products = {"apply": apply_products, "zhy": 10.0, "zipw": 10.0}
+        names = {"apply": apply_name, "zhy": "gemm2_kernel", "zipw": "zipw_tc_kernel"}
         sfx = f"config{args.config}" + ("_inversion" if args.inversion else "")
-        files = {"apply": ("k_contract_tc.cu", f"gemm1_kernel_{sfx}.md"),
+        files = {"apply": ("k_contract_tc.cu" if apply_products == 10.0 else "k_apply_mod.cu", f"{apply_name}_{sfx}.md"),
                  "zhy": ("k_contract_tc.cu", f"gemm2_kernel_{sfx}.md"),
                  "zipw": ("k_zipw_tc.cu", f"zipw_tc_kernel_{sfx}.md")}
         nlaunch_dom = st["n_batches"]
         if args.precision == "sliced":
             peak = peaks.get("bf16_tflops_sustained", 1700.0)
             # algorithmic flops of the kernel's step (the interstitial products by
-            # their FFT count); every real multiply-add expands into 10 BF16 slice products
+            # their FFT count); every real multiply-add expands into 10 BF16 slice products,
+            # or 4 residue products where the apply runs on residues
             alg = fl_fft if dom == "zipw" else kernels[dom][1]
-            achieved = 10.0 * alg / (kernels[dom][0] * 1e-3) / 1e12
+            achieved = products[dom] * alg / (kernels[dom][0] * 1e-3) / 1e12
             roof = {"bound": "tensor", "kernel": names[dom], "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": _profiled_traffic(*files[dom]),
                     "peak_source": f"bf16_tflops_sustained ({peak_kind})",
-                    "count": "10 BF16 slice products per real multiply-add of the algorithmic flops",
+                    "count": f"{products[dom]:.0f} BF16 products per real multiply-add of the algorithmic flops",
                     "algorithmic_flops_per_launch": alg / nlaunch_dom, "launches_per_step": nlaunch_dom,
                     "useful_tflops": alg / (kernels[dom][0] * 1e-3) / 1e12,
                     "per_kernel_ms": {names[k]: kernels[k][0] for k in kernels},
-                    "per_kernel_frac": {names[k]: 10.0 * (fl_fft if k == "zipw" else kernels[k][1]) /
+                    "per_kernel_frac": {names[k]: products[k] * (fl_fft if k == "zipw" else kernels[k][1]) /
                                         (kernels[k][0] * 1e-3) / 1e12 / peak for k in kernels if kernels[k][0] > 0},
                     "zipw_frac_direct_sum_count": 10.0 * kernels["zipw"][1] / (kernels["zipw"][0] * 1e-3) / 1e12 / peak
                     if kernels["zipw"][0] > 0 else None}
