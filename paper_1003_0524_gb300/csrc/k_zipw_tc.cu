@@ -531,12 +531,12 @@ __global__ void __launch_bounds__(256) ipw_transpose_kernel(const float4 *__rest
 // Band block: a multiple of 8 (the output width 2 NB is a multiple of 16) up to 64, the
 // one with the least padded bands times the time per padded band.  A narrow block reads
 // the 128 rows of A from shared memory for fewer columns; measured per band against 64
-// (2 atoms, 40 and 32 to 48 bands; 5 atoms, 120; 10 atoms, 250): 8: 3.1, 16: 1.74, 24:
-// 1.33, 32: 1.19, 40: 1.04 to 1.12, 48: 1.08, 56: 1.02.  (The least padding among 8 to
-// 40 took 24 for 48 bands, 70.1 ms against 57.3 with 48, and 32 for 250 bands, 7.5 ms
-// against 6.6 with 64.)
+// (5 atoms, 120 bands; 2 atoms, 40 bands): 8: 3.5 to 3.7, 16: 1.85 to 1.93, 24: 1.37 to
+// 1.39, 32: 1.20, 40: 1.12, 48: 1.07 to 1.09, 56: 1.01 to 1.04.  (The least padding among
+// 8 to 40 took 24 for 48 bands, 57.3 ms against 44.7 with 48, and 40 for 120 bands, 8.95
+// ms against 8.51 with 64.)
 int pick_nb(int nb_max) {
-    static const double per_band[8] = {3.1, 1.74, 1.33, 1.19, 1.06, 1.08, 1.02, 1.0};
+    static const double per_band[8] = {3.6, 1.89, 1.38, 1.2, 1.12, 1.08, 1.02, 1.0};
     int best = 8;
     double cost = 1e300;
     for (int nb = 8; nb <= 64; nb += 8) {
