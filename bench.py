@@ -64,10 +64,10 @@ def _profiled_traffic(kernel_file: str, profile: str):
 def _apply_kernel(s, st):
     """The kernel of the dense-block Coulomb apply and its tensor products per real
     multiply-add: 10 digit products, or, for complex dense blocks of 1280 to 6144 rows,
-    4 residue products (16 for a complex one: 8 moduli, 2 real products each)."""
+    4.5 residue products (18 for a complex one: 9 moduli, 2 real products each)."""
     n_lm = s.n_atoms * (s.Lmax + 1) ** 2
     D = max((n_lm if st["sparse_used"] else s.n_mt) + int(g.shape[0]) for g in s.Gaux)
-    return ("mod_gemm_kernel", 4.0) if not s.inversion and 1280 <= D <= 6144 else ("gemm1_kernel", 10.0)
+    return ("mod_gemm_kernel", 4.5) if not s.inversion and 1280 <= D <= 6144 else ("gemm1_kernel", 10.0)
 
 
 def _peaks():
@@ -433,13 +433,13 @@ def run_ours(args):
             peak = peaks.get("bf16_tflops_sustained", 1700.0)
             # algorithmic flops of the kernel's step (the interstitial products by
             # their FFT count); every real multiply-add expands into 10 BF16 slice products,
-            # or 4 residue products where the apply runs on residues
+            # or 4.5 residue products where the apply runs on residues
             alg = fl_fft if dom == "zipw" else kernels[dom][1]
             achieved = products[dom] * alg / (kernels[dom][0] * 1e-3) / 1e12
             roof = {"bound": "tensor", "kernel": names[dom], "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": _profiled_traffic(*files[dom]),
                     "peak_source": f"bf16_tflops_sustained ({peak_kind})",
-                    "count": f"{products[dom]:.0f} BF16 products per real multiply-add of the algorithmic flops",
+                    "count": f"{products[dom]:g} BF16 products per real multiply-add of the algorithmic flops",
                     "algorithmic_flops_per_launch": alg / nlaunch_dom, "launches_per_step": nlaunch_dom,
                     "useful_tflops": alg / (kernels[dom][0] * 1e-3) / 1e12,
                     "per_kernel_ms": {names[k]: kernels[k][0] for k in kernels},

@@ -1,24 +1,30 @@
 // k_apply_mod.cu -- the Coulomb apply Y' = U Z of large dense blocks as exact integer
-// products modulo eight small numbers (tcgen05.mma kind::f16 with BF16 operands).
+// products modulo nine small numbers (tcgen05.mma kind::f16 with BF16 operands).
 //
 // Every row of U (the dense-block rows of the upper triangle of v_t with half its
 // diagonal) and every column of Z is scaled by a power of two and rounded to complex
-// integers a, b of Euclidean norm below 2^35.04.  Then |Re|, |Im| of sum_k a_k b_k stay
-// below M / 2 for M = m_1 ... m_8 = 2^71.08, and the sum is known exactly from its
+// integers a, b of Euclidean norm below 2^39.39.  Then |Re|, |Im| of sum_k a_k b_k stay
+// below M / 2 for M = m_1 ... m_9 = 2^79.79, and the sum is known exactly from its
 // residues modulo the m_i (Chinese remainder theorem).  Modulo m, a product of primes
 // = 1 mod 4, there is a j with j^2 = -1, and x + i y -> (x + j y, x - j y) turns one
-// complex product into two real ones.  So a complex product costs 16 real products of
-// residues |r| <= 254, instead of the 40 of the digit scheme (ten digit products for
+// complex product into two real ones.  So a complex product costs 18 real products of
+// residues |r| <= 255, instead of the 40 of the digit scheme (ten digit products for
 // each of the four real products of the embedding [[Re, -Im], [Im, Re]]).
 //
 // A residue is an integer of at most 8 bits, exact in BF16; a product sum over 256 K
 // values stays below 2^24 and is exact in the FP32 accumulators, after which the
 // accumulator is reduced modulo m on the CUDA cores and added up as a small integer.
-// The only error is the rounding of the operands: 0.3 units against components of
-// about 2^29 units (2660 functions), 2^-30 relative, below that of the digits (which
-// drop the products of weight 2^-48 and less).
+// The only error is the rounding of the operands, whose units are at most 2^-38.39 of
+// the line's norm.  The norm is at most sqrt(2 D) times the largest component, so up to
+// 6144 functions a unit is at most 2^-31.6 of that component, however the line is
+// distributed, where the digits have 2^-32 to 2^-31 of it and drop products besides.
+// Error of Y' over its largest element, D = 1280, 2660, 6144, by a model of both
+// roundings: elements of equal size 4e-11, 5e-11, 9e-11 (digits 1e-10 at each), Gaussian
+// 5e-11, 5e-11, 9e-11 (1.4e-9, 1.8e-9, 1.9e-9), decaying 4e-12 (5e-9 to 1e-8).  Eight
+// moduli (norms below 2^35.04) were 11 % fewer products, but at equal size 7e-10, 1.9e-9,
+// 1.4e-9, above the digits.
 //
-// The residues of Z and of Y' take 32 bytes per complex element each (the digits of Z
+// The residues of Z and of Y' take 36 bytes per complex element each (the digits of Z
 // and Y' in FP64 16 each), so the scheme pays where the products outweigh the extra
 // traffic; apply_mod_usable holds the rule and its figures.
 #include <algorithm>
@@ -34,9 +40,9 @@ using namespace tc;
 namespace {
 
 // ------------------------------------------------------------- moduli
-constexpr int NM = 8, NC16 = 2 * NM;                      // moduli; residue planes (x + j y, x - j y per modulus)
-constexpr int kMod[NM] = {509, 505, 493, 481, 461, 457, 449, 433};
-constexpr float kHalfBits = 35.04f;                       // (log2 M - 1) / 2, rounded down
+constexpr int NM = 9, NRP = 2 * NM;                       // moduli; residue planes (x + j y, x - j y per modulus)
+constexpr int kMod[NM] = {509, 505, 493, 481, 461, 457, 449, 433, 421};
+constexpr float kHalfBits = 39.399f;                      // (log2 M - 1) / 2 = 39.39907, rounded down
 
 constexpr int mod_root(int m) {
     for (int j = 1; j < m; ++j)
@@ -75,8 +81,8 @@ constexpr unsigned long long frac64(int c, int m) {
 }
 struct ModTab {
     float m[NM] = {}, inv[NM] = {};                       // modulus and its reciprocal
-    float c12[NM] = {}, c24[NM] = {};                     // 2^12, 2^24 mod m
-    float d0[NM] = {}, d12[NM] = {}, d24[NM] = {};        // j, j 2^12, j 2^24 mod m
+    float c13[NM] = {}, c26[NM] = {};                     // 2^13, 2^26 mod m
+    float d0[NM] = {}, d13[NM] = {}, d26[NM] = {};        // j, j 2^13, j 2^26 mod m
     // x mod M = M frac(sum_i (p_i + q_i) re_i), y = M frac(sum_i (p_i - q_i) im_i): 64-bit
     // fractions, the low word as a signed number
     int re_lo[NM] = {}, im_lo[NM] = {};
@@ -88,11 +94,11 @@ constexpr ModTab make_tab() {
         const int m = kMod[i], j = mod_root(m), oi = mod_inv(others(i), m);
         t.m[i] = (float)m;
         t.inv[i] = 1.0f / (float)m;
-        t.c12[i] = (float)balanced(1LL << 12, m);
-        t.c24[i] = (float)balanced(1LL << 24, m);
+        t.c13[i] = (float)balanced(1LL << 13, m);
+        t.c26[i] = (float)balanced(1LL << 26, m);
         t.d0[i] = (float)balanced(j, m);
-        t.d12[i] = (float)balanced((long long)j << 12, m);
-        t.d24[i] = (float)balanced((long long)j << 24, m);
+        t.d13[i] = (float)balanced((long long)j << 13, m);
+        t.d26[i] = (float)balanced((long long)j << 26, m);
         const unsigned long long wr = frac64((int)((long long)mod_inv(2, m) * oi % m), m);
         const unsigned long long wi = frac64((int)((long long)mod_inv(2 * j % m, m) * oi % m), m);
         t.re_lo[i] = (int)(unsigned)wr;
@@ -103,33 +109,36 @@ constexpr ModTab make_tab() {
     return t;
 }
 __constant__ ModTab kTab = make_tab();
-// U is scaled by kKappa = M / 2^71 besides its power of two, so that a result is its
-// 64-bit fraction times a power of two
-constexpr double kKappa = mod_product() / 2361183241434822606848.0;
+// U is scaled by kKappa = M / 2^79 besides its power of two, so that a result is its
+// 64-bit fraction times a power of two, 2^kFracExp for operands of scale 1
+constexpr double kKappa = mod_product() / 604462909807314587353088.0;
+constexpr int kFracExp = 79 - 64;
 
 // ------------------------------------------------------------- residues
 __device__ __forceinline__ uint64_t f2_both(float x) { return f2_pack(__float_as_uint(x), __float_as_uint(x)); }
 
-// round(|x| 2^s) with the sign of x, for |x| 2^s < 2^36 (0 for zeros and subnormals),
-// as three 12-bit pieces x = p2 2^24 + p1 2^12 + p0, |p0|, |p1| <= 2048, |p2| <= 2107
+// |N| < 2^39.4 as three pieces N = p2 2^26 + p1 2^13 + p0, |p0|, |p1| <= 4096,
+// |p2| < 10810
 __device__ __forceinline__ void pieces_of(long long N, float (&p)[3]) {
-    const unsigned long long v = (unsigned long long)N + 0x800800800ULL;
+    const unsigned long long v = (unsigned long long)N + 0x2001000ULL;   // 2^25 + 2^12
     const uint32_t vl = (uint32_t)v, vh = (uint32_t)(v >> 32);
-    p[0] = __uint_as_float(0x4B000000u | (vl & 0xfffu)) - 8390656.0f;
-    p[1] = __uint_as_float(0x4B000000u | ((vl >> 12) & 0xfffu)) - 8390656.0f;
-    p[2] = __int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 24)) - 12584960.0f;
+    p[0] = __uint_as_float(0x4B000000u | (vl & 0x1fffu)) - 8392704.0f;
+    p[1] = __uint_as_float(0x4B000000u | ((vl >> 13) & 0x1fffu)) - 8392704.0f;
+    p[2] = __int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 26)) - 12582912.0f;
 }
+// The pieces of round(|x| 2^s) with the sign of x (0 for zeros and subnormals)
 __device__ __forceinline__ void int_pieces(double x, int s, float (&p)[3]) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
     const int E = (int)((hi >> 20) & 0x7ffu);
-    const int sh = E ? max(1074 - E - s, 0) : 64;         // one bit below the unit; >= 16 by |x| 2^s < 2^36
+    const int sh = E ? max(1074 - E - s, 0) : 64;         // one bit below the unit; >= 12 by |x| 2^s < 2^40
     const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
     const unsigned long long q = ((sh < 64 ? m >> sh : 0ULL) + 1) >> 1;
     const unsigned long long neg = (unsigned long long)((long long)(int)hi >> 63);
     pieces_of((long long)((q ^ neg) - neg), p);
 }
 
-// p - m round(p / m) for packed integers |p| < 2^22
+// p - m round(p / m) for packed integers |p| < 2^24: at most 255 (the rounding of p / m may
+// miss the nearest integer by 0.002)
 __device__ __forceinline__ uint64_t f2_reduce(uint64_t p, int i) {
     const uint64_t magic = f2_both(12582912.0f);
     const uint64_t k = f2_sub(f2_fma(p, f2_both(kTab.inv[i]), magic), magic);
@@ -138,10 +147,10 @@ __device__ __forceinline__ uint64_t f2_reduce(uint64_t p, int i) {
 __device__ __forceinline__ uint32_t f2_bf16(uint64_t v) { return __byte_perm((uint32_t)v, (uint32_t)(v >> 32), 0x7632); }
 
 // The residues of two complex integers (packed pieces) modulo m_i as BF16 pairs:
-// x + j y and x - j y.
+// x + j y and x - j y, from sums below 254 (10810 + 4096 + 1) + 254 (10810 + 2 4096) < 2^23.1.
 __device__ __forceinline__ void residues(const uint64_t (&X)[3], const uint64_t (&Y)[3], int i, uint32_t &plus, uint32_t &minus) {
-    const uint64_t a = f2_fma(X[2], f2_both(kTab.c24[i]), f2_fma(X[1], f2_both(kTab.c12[i]), X[0]));
-    const uint64_t b = f2_fma(Y[2], f2_both(kTab.d24[i]), f2_fma(Y[1], f2_both(kTab.d12[i]), f2_mul(Y[0], f2_both(kTab.d0[i]))));
+    const uint64_t a = f2_fma(X[2], f2_both(kTab.c26[i]), f2_fma(X[1], f2_both(kTab.c13[i]), X[0]));
+    const uint64_t b = f2_fma(Y[2], f2_both(kTab.d26[i]), f2_fma(Y[1], f2_both(kTab.d13[i]), f2_mul(Y[0], f2_both(kTab.d0[i]))));
     plus = f2_bf16(f2_reduce(f2_add(a, b), i));
     minus = f2_bf16(f2_reduce(f2_sub(a, b), i));
 }
@@ -175,7 +184,7 @@ struct SquareSum {
         if (ref > r2) o.rescale(ref);
         s += o.s;
     }
-    // power of two that takes the norm just below 2^35.04 (margins: the truncation of
+    // power of two that takes the norm just below 2^bits (margins: the truncation of
     // part(), the FP32 sum, the rounding of up to 2 x 6144 components to integers)
     __device__ __forceinline__ int scale(float bits) const {
         if (!(s > 0.0f)) return 0;
@@ -244,9 +253,9 @@ __global__ void __launch_bounds__(256) mod_u_kernel(const double2 *__restrict__ 
 // apply), from the interstitial rows (F32: the interstitial kernel's plane ZI [g][col] of
 // FP32 pairs in units of 2^cexp[col]; else Z itself, where a caller's projections are in
 // it) and the muffin-tin rows of Z; the layout and the passes of slice_z_kernel, with the
-// sum of squares of the dense rows beside the maximum.  Bound by memory: 32 bytes read, 48 written per element.
+// sum of squares of the dense rows beside the maximum.  Bound by memory: 32 bytes read, 52 written per element.
 constexpr int MZ_COLS = 8, MZ_THREADS = 256, MZ_NJ = MZ_THREADS / MZ_COLS, MZ_CH = 4 * MZ_NJ, MZ_CS = MZ_CH + 8;
-constexpr size_t kMzSmem = (size_t)(2 * NPL + NC16) * MZ_COLS * MZ_CS * sizeof(__nv_bfloat16);
+constexpr size_t kMzSmem = (size_t)(2 * NPL + NRP) * MZ_COLS * MZ_CS * sizeof(__nv_bfloat16);
 template <bool F32>
 __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const float4 *__restrict__ ZI, long long NCi,
                                                            const int *__restrict__ cexp,
@@ -370,7 +379,7 @@ __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const float4 *__re
         }
         if (u0 + CH < uend) fetch(u0 + CH + 4 * j);   // the next chunk, while this one is stored
         __syncthreads();
-        const int nplane = u0 + CH > N0pad ? 2 * NPL + NC16 : 2 * NPL;
+        const int nplane = u0 + CH > N0pad ? 2 * NPL + NRP : 2 * NPL;
         for (int t = tid; t < nplane * MZ_COLS * (CH / 8); t += MZ_THREADS) {
             const int x = t % (CH / 8), line = t / (CH / 8), cc = line % MZ_COLS, pp = line / MZ_COLS, u = u0 + 8 * x;
             if (c0 + cc >= q.ncols) continue;
@@ -495,7 +504,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(M_THREADS, 1)
             int4 tl;
             while (!abort_flag && walk.next(tl, plane)) {
                 const int yz = (int)(plane * p.NC) + tl.z + rank * (M_BM / 2);
-                const int yu = (tl.x * NC16 + plane) * p.Dp + mt_row0(tl) + rank * 64;
+                const int yu = (tl.x * NRP + plane) * p.Dp + mt_row0(tl) + rank * 64;
                 const int nchunk = mt_chunks(tl);
                 bool stop = false;
                 for (int kc = 0; kc < nchunk; ++kc) {
@@ -672,8 +681,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(M_THREADS, 1)
 // From the residues of Y' (dense rows) and the FP64 mu = 0 rows Y0 [col][N0] to the digits
 // of Y' for Z^H Y.  One block per column: the values F 2^e of the dense rows (F: the 64-bit
 // fraction of the residues, see ModTab) stay in shared memory between the pass that finds
-// the column's exponent and the one that cuts the digits.  Bound by memory: 32 bytes
-// read and 16 written per element, and the ~100 integer operations of an element.
+// the column's exponent and the one that cuts the digits.  Bound by memory: 36 bytes
+// read and 16 written per element, and the ~110 integer operations of an element.
 constexpr int MY_THREADS = 256;
 __device__ __forceinline__ int bit_length(long long f) { return 64 - __clzll(f < 0 ? -f : f); }
 
@@ -745,7 +754,7 @@ __global__ void __launch_bounds__(MY_THREADS) mod_y_kernel(const short *__restri
                 f.y = (long long)((unsigned long long)li[t] + ((unsigned long long)hi[t] << 32));
                 val[t * ng + g] = f;
                 if (4 * g + t < q.D && (f.x | f.y))
-                    emax = max(emax, max(bit_length(f.x), bit_length(f.y)) + 7 - ue[4 * g + t] - sb);
+                    emax = max(emax, max(bit_length(f.x), bit_length(f.y)) + kFracExp - ue[4 * g + t] - sb);
             }
         }
 #pragma unroll
@@ -766,7 +775,7 @@ __global__ void __launch_bounds__(MY_THREADS) mod_y_kernel(const short *__restri
                     // (dr and t: N0pad is a multiple of 4, so row dr sits at [t][(u - N0pad) / 4])
                     const bool in = dr < q.D;
                     const longlong2 f = in ? val[t * ng + (u - N0pad) / 4] : make_longlong2(0, 0);
-                    const int x = in ? 7 - ue[dr] - sb + 32 - e : 0;
+                    const int x = in ? kFracExp - ue[dr] - sb + 32 - e : 0;
                     sr[t] = slice_i64(f.x, x);
                     si[t] = slice_i64(f.y, x);
                 } else {
@@ -800,8 +809,8 @@ ModSizes apply_mod_sizes(int maxD) {
     ModSizes z;
     z.Kp = (maxD + M_KB - 1) / M_KB * M_KB;
     z.Dp = (maxD + M_BN - 1) / M_BN * M_BN;
-    z.u_elems = (size_t)NC16 * z.Dp * z.Kp;
-    z.col_bytes = (size_t)NC16 * z.Kp * 2;
+    z.u_elems = (size_t)NRP * z.Dp * z.Kp;
+    z.col_bytes = (size_t)NRP * z.Kp * 2;
     return z;
 }
 
@@ -824,7 +833,7 @@ int apply_mod_tiles(const QDesc *h_q, int nq, std::vector<unsigned char> &out) {
                     if (c < cend) tiles.push_back(make_int4(q.iq, r | ((kend - r) / M_KC) << 16, (int)c, (int)cend));
                 }
     }
-    if (tiles.size() > (size_t)0x7fffffff / NC16) return -1;
+    if (tiles.size() > (size_t)0x7fffffff / NRP) return -1;
     out.assign(reinterpret_cast<const unsigned char *>(tiles.data()),
                reinterpret_cast<const unsigned char *>(tiles.data()) + tiles.size() * sizeof(int4));
     return (int)tiles.size();
@@ -848,18 +857,18 @@ int apply_mod_slice_z(hfx_ctx *ctx, const float4 *d_ZI, const int *d_cexp, const
 int apply_mod_run(hfx_ctx *ctx, const __nv_bfloat16 *d_UR_all, int nk, const __nv_bfloat16 *d_ZR, short *d_YR, long long NC,
                   const ModSizes &z, const void *d_tiles, int nplane) {
     if (nplane == 0) return HFX_OK;
-    if (NC > 0x7fffffffLL / NC16 || (long long)nk * NC16 * z.Dp > 0x7fffffffLL)
+    if (NC > 0x7fffffffLL / NRP || (long long)nk * NRP * z.Dp > 0x7fffffffLL)
         return set_err(ctx, HFX_EUNSUPPORTED, "batch has too many columns for 32-bit TMA coordinates");
     int rc;
     CUtensorMap mZ, mU, mY;
-    if ((rc = make_map_2d_sw(ctx, &mZ, d_ZR, (long long)NC16 * NC, z.Kp, M_BM / 2, M_KB, 128)) ||
-        (rc = make_map_2d_sw(ctx, &mU, d_UR_all, (long long)nk * NC16 * z.Dp, z.Kp, 64, M_KB, 128)) ||
-        (rc = make_map_2d_sw(ctx, &mY, d_YR, (long long)NC16 * NC, z.Kp, 32, 64, 128)))
+    if ((rc = make_map_2d_sw(ctx, &mZ, d_ZR, (long long)NRP * NC, z.Kp, M_BM / 2, M_KB, 128)) ||
+        (rc = make_map_2d_sw(ctx, &mU, d_UR_all, (long long)nk * NRP * z.Dp, z.Kp, 64, M_KB, 128)) ||
+        (rc = make_map_2d_sw(ctx, &mY, d_YR, (long long)NRP * NC, z.Kp, 32, 64, 128)))
         return rc;
     MParams p;
     p.tiles = reinterpret_cast<const int4 *>(d_tiles);
     p.nplane = nplane;
-    p.ntiles = nplane * NC16;
+    p.ntiles = nplane * NRP;
     p.Dp = z.Dp;
     p.Kp = z.Kp;
     p.NC = NC;
