@@ -63,11 +63,11 @@ def _profiled_traffic(kernel_file: str, profile: str):
 
 def _apply_kernel(s, st):
     """The kernel of the dense-block Coulomb apply and its tensor products per real
-    multiply-add: 10 digit products, or, for complex dense blocks of 1280 to 6144 rows,
+    multiply-add: 10 digit products, or, for complex dense blocks of 1664 to 6144 rows,
     4.5 residue products (18 for a complex one: 9 moduli, 2 real products each)."""
     n_lm = s.n_atoms * (s.Lmax + 1) ** 2
     D = max((n_lm if st["sparse_used"] else s.n_mt) + int(g.shape[0]) for g in s.Gaux)
-    return ("mod_gemm_kernel", 4.5) if not s.inversion and 1280 <= D <= 6144 else ("gemm1_kernel", 10.0)
+    return ("mod_gemm_kernel", 4.5) if not s.inversion and 1664 <= D <= 6144 else ("gemm1_kernel", 10.0)
 
 
 def _peaks():

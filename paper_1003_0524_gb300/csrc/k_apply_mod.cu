@@ -799,11 +799,19 @@ __global__ void __launch_bounds__(MY_THREADS) mod_y_kernel(const short *__restri
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// From 1280 dense functions on: at 1225 (5 atoms, 120 bands, 8 k) the products take 3.3 ms
-// instead of 5.9, but the residues 2.7 ms more than the digits and FP64 values (20.1 against
-// 19.9 ms for the build); at 2660 (10 atoms, one k) 7.9 instead of 16.8 ms, with 3.0 ms more
-// (28.8 against 34.8 ms).  Up to 6144: a column's 64-bit values have to fit shared memory.
-bool apply_mod_usable(int maxD) { return maxD >= 1280 && maxD <= 6144; }
+// From 1664 dense functions on.  Builds with residues and with digits, ms:
+//   functions        1285         1425         1625         1825         2025
+//   8 k, 120 bands   20.4 / 18.7  21.9 / 20.7  24.6 / 24.4  28.2 / 28.5  30.2 / 32.2
+//   8 k, 40 bands    3.62 / 3.47                            4.82 / 4.96
+// (20 and 8 bands occupied: 154000 and 20500 columns; the products take 0.65 to 0.75 of
+// those of the digits from 1425 on, the extra residues grow with the size alone), and
+//   functions               1285         1625         1925         2425         6125
+//   one k, 4800 columns     3.05 / 3.04  3.57 / 3.57  4.17 / 4.15  5.14 / 5.33  13.1 / 14.4
+//   one k, 320 columns      0.80 / 0.81  0.92 / 0.92  1.01 / 1.03  1.17 / 1.21  2.56 / 2.69
+// Few columns do not change the line much: below it they lose up to 0.03 ms (48 columns:
+// 0.48 / 0.50 at 1285).  Up to 6144, where the unit of the residues still is no larger
+// than the largest one of the digits (2^-31 of a line's largest element, see above).
+bool apply_mod_usable(int maxD) { return maxD >= 1664 && maxD <= 6144; }
 
 ModSizes apply_mod_sizes(int maxD) {
     ModSizes z;

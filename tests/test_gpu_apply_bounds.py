@@ -2,12 +2,12 @@
 projections (GB300 only).  One band is a column z of such elements, the others are unit
 vectors of the first functions, so that V^x holds single elements of U z (U the upper
 triangle): no sum of Z^H Y hides the error of the apply.  Both sides of the limits between
-digits and residues (1280 and 6144 dense functions), against the sums in FP64.
+digits and residues (1664 and 6144 dense functions), against the sums in FP64.
 
 Tolerance on the root mean square over 128 components: the operands of the residue apply
 are rounded to units of at most 2^-38.39 of their line's norm, a sqrt(2 D) for D elements
 a (+-1 +- i); the 4 D independent errors of a component add up to the standard deviation
-2 D 2^-38.39 a b / sqrt 6 (both operands).  Those of the digits are smaller at D = 1279.
+2 D 2^-38.39 a b / sqrt 6 (both operands).  Those of the digits are smaller at D = 1663.
 The digits of U z that Z^H Y reads have units of 2^(e-32), e the column's exponent.  The
 mean square of 128 samples scatters by 6 % (one standard deviation, root): 1.4 is six.
 """
@@ -22,7 +22,7 @@ from paper_1003_0524_gb300 import synthetic as S
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("D", [1279, 1280, 2660, 6144, 6145])
+@pytest.mark.parametrize("D", [1663, 1664, 2660, 6144, 6145])
 def test_lines_of_equal_magnitude(D):
     import torch
     if not torch.cuda.is_available():
