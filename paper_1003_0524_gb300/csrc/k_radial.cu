@@ -7,7 +7,7 @@
 //   - the overlap matrix of the products and its largest eigenpairs;
 //     eigenfunctions with eigenvalue above the threshold are linearly
 //     independent, and the P largest of them (L = 0: P - 1 after the constant)
-//     become the functions M_aLP, normalised, each with its largest eigenvector
+//     become the functions M_aLP, orthonormal, each with its largest eigenvector
 //     component positive;
 //   - the multipole moments mu_aLP = int M r^(L+2) dr (Sec. III.C), the radial
 //     integrals R = int M u_lp u_l'p' r^2 dr, and the on-site Coulomb integrals
@@ -433,6 +433,48 @@ __global__ void __launch_bounds__(RP_THREADS) radial_functions_kernel(int n_r, c
     if (i < n_r) M[((size_t)L * P + Pi) * n_r + i] = v;
 }
 
+// The functions of one L made orthonormal on the grid, in descending order of the
+// eigenvalue (one block per L).  An eigenvector is accurate to rounding in the norm of
+// the overlap matrix, so what it holds of one with a larger eigenvalue grows by the root
+// of their ratio once it is scaled by 1/sqrt(eigenvalue): overlaps of the functions
+// reached 4e-12 at lmax 8, 1e-15 here.  The overlaps G = K K^T (Cholesky), a warp each,
+// then M = K^-1 M: 0.504 to 0.520 ms for the whole call at lmax 4, P = 3, 600 points.
+constexpr int RO_THREADS = 512;
+__global__ void __launch_bounds__(RO_THREADS) radial_orthonormal_kernel(int n_r, const double *__restrict__ r,
+                                                                        const double *__restrict__ w, int P,
+                                                                        const int *__restrict__ status,
+                                                                        double *__restrict__ M) {
+    if (*status < 0) return;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    __shared__ double K[kMaxP][kMaxP + 1];   // lower triangle; the diagonal inverted
+    double *ML = M + (size_t)blockIdx.x * P * n_r;
+    for (int t = warp; t < P * (P + 1) / 2; t += RO_THREADS / 32) {
+        int a = 0, b = t;
+        while (b > a) { b -= a + 1; ++a; }
+        const double *x = ML + (size_t)a * n_r, *y = ML + (size_t)b * n_r;
+        double s = 0.0;
+#pragma unroll 8
+        for (int i = lane; i < n_r; i += 32) s = fma(w[i] * r[i] * r[i] * x[i], y[i], s);
+        s = warp_sum(s);
+        if (lane == 0) K[a][b] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int a = 0; a < P; ++a)
+            for (int b = 0; b <= a; ++b) {
+                double s = K[a][b];
+                for (int j = 0; j < b; ++j) s = fma(-K[a][j], K[b][j], s);
+                K[a][b] = a == b ? 1.0 / sqrt(s) : s * K[b][b];
+            }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_r; i += RO_THREADS)
+        for (int a = 0; a < P; ++a) {
+            double v = ML[(size_t)a * n_r + i];
+            for (int j = 0; j < a; ++j) v = fma(-K[a][j], ML[(size_t)j * n_r + i], v);
+            ML[(size_t)a * n_r + i] = v * K[a][a];
+        }
+}
+
 // r^k, k >= 0
 __device__ __forceinline__ double ipow(double r, int k) {
     double p = 1.0;
@@ -643,6 +685,7 @@ int hfx_set_radial_functions(hfx_ctx *ctx, int atom, int n_r, const double *r, c
     radial_eigen_kernel<<<nL, RE_THREADS, sm, st>>>(dp(o_O), d_nc, maxc, nL, P, threshold, dp(o_V), d_status);
     radial_functions_kernel<<<dim3((n_r + RP_THREADS - 1) / RP_THREADS, P, nL), RP_THREADS, 0, st>>>(
         n_r, d_r, d_w, dp(o_f), dp(o_V), d_nc, maxc, P, d_status, dM);
+    radial_orthonormal_kernel<<<nL, RO_THREADS, 0, st>>>(n_r, d_r, d_w, P, d_status, dM);
     const long long nint = (long long)LP * (1 + nlp * (nlp + 1) / 2);
     radial_integrals_kernel<<<(unsigned)((nint + RP_THREADS / 32 - 1) / (RP_THREADS / 32)), RP_THREADS, 0, st>>>(
         n_r, d_r, d_w, d_u, dM, nlp, P, nL, d_status, dmu, dR);
