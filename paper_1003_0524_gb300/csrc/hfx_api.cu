@@ -55,6 +55,12 @@ void dfree(void *p) {
     if (p) cudaFree(p);
 }
 
+void release(Scratch &s) {
+    dfree(s.p);
+    s.p = nullptr;
+    s.bytes = 0;
+}
+
 template <typename T> int h2d(hfx_ctx *ctx, T *dst, const T *src, size_t n) {
     if (n == 0) return HFX_OK;
     return cuda_check(ctx, cudaMemcpyAsync(dst, src, n * sizeof(T), cudaMemcpyHostToDevice, ctx->stream), "copy to device");
@@ -105,6 +111,58 @@ int check_inversion_bands(hfx_ctx *ctx, int ik, int nb, int npw, const double *c
     if (dev > ctx->opt.herm_tol * std::max(amax, 1e-300))
         return set_err(ctx, HFX_EINVAL, "set_kpoint: MT coefficients do not satisfy phi(-r) = phi(r)^* (inversion mode)");
     return HFX_OK;
+}
+
+// The checks of set_coulomb on the host; magnitudes are compared by their bits, so that
+// one vectorised pass finds the largest one and what is not finite.
+void check_coulomb_host(const double *v, int n, size_t ld, CoulombCheck *chk) {
+    unsigned long long mr = 0, mi = 0;
+    for (int i = 0; i < n; ++i) {
+        const double *row = v + 2 * (size_t)i * ld;
+        for (int j = 0; j < n; ++j) {
+            unsigned long long r, m;
+            std::memcpy(&r, row + 2 * j, 8);
+            std::memcpy(&m, row + 2 * j + 1, 8);
+            mr = std::max(mr, r & 0x7fffffffffffffffULL);
+            mi = std::max(mi, m & 0x7fffffffffffffffULL);
+        }
+    }
+    chk->mx = std::max(mr, mi);
+    chk->im = mi;
+    chk->nonfinite = chk->mx >= 0x7ff0000000000000ULL;
+    double dev = 0.0;
+    for (int i = 0; i < n && !chk->nonfinite; ++i)
+        for (int j = 0; j <= i; ++j) {
+            const double *a = v + 2 * ((size_t)i * ld + j), *b = v + 2 * ((size_t)j * ld + i);
+            dev = std::max(dev, std::fabs(a[0] - b[0]) + std::fabs(a[1] + b[1]));
+        }
+    std::memcpy(&chk->dev, &dev, 8);
+}
+// Above this many functions the check runs on the device, whose two more copies and
+// launches cost a small call more than they save.  A call at 51, 80, 128, 144, 160 and 190
+// functions: 21, 31, 51, 57, 69, 90 us with the check on the host, 52, 55, 57, 57, 58, 60
+// with that on the device.
+constexpr int kHostCheckMax = 144;
+
+// Device memory for a v that is being checked beside the one it replaces: a build buffer
+// where one is large enough (their contents are dead outside a build), the slices of U
+// (which the next build then makes anew), else a buffer of its own that the next build
+// gives back; null if there is no memory.
+double2 *coulomb_stage(hfx_ctx *ctx, size_t bytes) {
+    for (Scratch *b : {&ctx->s_zc, &ctx->s_zs, &ctx->s_ys, &ctx->s_vin})
+        if (b->bytes >= bytes) return reinterpret_cast<double2 *>(b->p);
+    if (ctx->s_ap.bytes >= bytes) {
+        ctx->coulomb_dirty = true;
+        return reinterpret_cast<double2 *>(ctx->s_ap.p);
+    }
+    release(ctx->s_vin);
+    if (cudaMalloc(&ctx->s_vin.p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->s_vin.p = nullptr;
+        return nullptr;
+    }
+    ctx->s_vin.bytes = bytes;
+    return reinterpret_cast<double2 *>(ctx->s_vin.p);
 }
 
 long long rup(long long x, long long m) { return (x + m - 1) / m * m; }
@@ -400,43 +458,75 @@ int hfx_set_coulomb(hfx_ctx *ctx, int iq, int n_ipw, const int *G_aux, const dou
     const int naux = ctx->nmt + n_ipw;
     if (ld < naux) return set_err(ctx, HFX_EINVAL, "set_coulomb: leading dimension below N_aux");
     const size_t nv = (size_t)naux * naux;
-    // v goes to a staging buffer of the context, is checked there on the device (three
-    // host passes over the matrix took four fifths of this call) and copied to its
-    // place only when it passes: a refused v leaves the one before it as it was
     int rc = cuda_check(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
     if (rc) return rc;
-    if ((rc = scratch_reserve(ctx, ctx->s_qd, nv * sizeof(double2) + sizeof(CoulombCheck)))) return rc;
-    double2 *d_in = reinterpret_cast<double2 *>(ctx->s_qd.p);
-    CoulombCheck *d_chk = reinterpret_cast<CoulombCheck *>(d_in + nv), chk;
-    if ((rc = cuda_check(ctx, cudaMemcpy2DAsync(d_in, 16 * (size_t)naux, v, 16 * (size_t)ld, 16 * (size_t)naux, naux,
-                                                cudaMemcpyHostToDevice, ctx->stream), "copy to device")))
-        return rc;
-    launch_check_coulomb(d_in, naux, ctx->opt.inversion ? 1 : 0, d_chk, ctx->stream);
-    if ((rc = cuda_check(ctx, cudaGetLastError(), "set_coulomb check")) ||
-        (rc = cuda_check(ctx, cudaMemcpyAsync(&chk, d_chk, sizeof(chk), cudaMemcpyDeviceToHost, ctx->stream), "set_coulomb check")) ||
-        (rc = sync(ctx)))
-        return rc;
-    if (chk.nonfinite) return set_err(ctx, HFX_ENONFINITE, "set_coulomb: non-finite element");
+    QPoint &q = ctx->qp[iq];
+    const bool first = !q.set;
+    auto place = [&]() {
+        int e;
+        dfree(q.d_G); dfree(q.d_v);
+        q.d_G = nullptr; q.d_v = nullptr;
+        if ((e = dalloc(ctx, &q.d_G, (size_t)3 * std::max(n_ipw, 1))) == HFX_OK) e = dalloc(ctx, &q.d_v, nv);
+        return e;
+    };
+    // Small matrices are checked on the host; others on the device: the first v of a q in
+    // its place, a later one beside it, so that a refused v leaves the one before it as it
+    // was (on the host where there is no memory for that).  q is set again only at the end
+    double2 *d_in = nullptr;
+    if (naux > kHostCheckMax) {
+        if (first && (rc = place())) return rc;
+        d_in = first ? q.d_v : coulomb_stage(ctx, nv * sizeof(double2));
+    }
+    if ((d_in || ctx->opt.inversion) && (rc = scratch_reserve(ctx, ctx->s_chk, sizeof(CoulombCheck)))) return rc;
+    CoulombCheck *d_chk = reinterpret_cast<CoulombCheck *>(ctx->s_chk.p), chk;
+    auto upload = [&](double2 *d) {
+        // (one copy is faster up to some MB, rows are from some 10 MB on)
+        if (ld == naux && !d_in) return h2d(ctx, d, reinterpret_cast<const double2 *>(v), nv);
+        return cuda_check(ctx, cudaMemcpy2DAsync(d, 16 * (size_t)naux, v, 16 * (size_t)ld, 16 * (size_t)naux, naux,
+                                                 cudaMemcpyHostToDevice, ctx->stream), "copy to device");
+    };
+    if (d_in) {
+        if ((rc = upload(d_in))) return rc;
+        launch_check_coulomb(d_in, naux, ctx->opt.inversion ? 1 : 0, d_chk, ctx->stream);
+        if ((rc = cuda_check(ctx, cudaGetLastError(), "set_coulomb check")) ||
+            (rc = cuda_check(ctx, cudaMemcpyAsync(&chk, d_chk, sizeof(chk), cudaMemcpyDeviceToHost, ctx->stream), "set_coulomb check")) ||
+            (rc = sync(ctx)))
+            return rc;
+    } else {
+        check_coulomb_host(v, naux, ld, &chk);
+    }
     double mx, dev, im;
     std::memcpy(&mx, &chk.mx, 8);
     std::memcpy(&dev, &chk.dev, 8);
     std::memcpy(&im, &chk.im, 8);
     const double tol = ctx->opt.herm_tol * std::max(mx, 1e-300);
-    if (dev > tol) return set_err(ctx, HFX_ENOTHERM, "set_coulomb: v(q) is not Hermitian");
+    if (chk.nonfinite) rc = set_err(ctx, HFX_ENONFINITE, "set_coulomb: non-finite element");
+    else if (dev > tol) rc = set_err(ctx, HFX_ENOTHERM, "set_coulomb: v(q) is not Hermitian");
     // over the symmetrized MT functions of Sec. III.D, v(q) is real
-    if (ctx->opt.inversion && im > tol)
-        return set_err(ctx, HFX_EINVAL, "set_coulomb: v(q) over the symmetrized basis is not real (inversion mode)");
-    QPoint &q = ctx->qp[iq];
-    if (q.set && q.nipw != n_ipw) {
-        dfree(q.d_G); dfree(q.d_v); dfree(q.d_VD); dfree(q.d_VB);
-        q.d_G = nullptr; q.d_v = nullptr; q.d_VD = nullptr; q.d_VB = nullptr;
-        q.vd_cap = q.vb_cap = 0;
+    else if (ctx->opt.inversion && im > tol)
+        rc = set_err(ctx, HFX_EINVAL, "set_coulomb: v(q) over the symmetrized basis is not real (inversion mode)");
+    if (rc) {
+        if (first && d_in) { dfree(q.d_v); q.d_v = nullptr; }
+        return rc;
     }
-    if (!q.d_v && ((rc = dalloc(ctx, &q.d_G, (size_t)3 * std::max(n_ipw, 1))) || (rc = dalloc(ctx, &q.d_v, nv))))
-        return rc;
-    if ((rc = h2d(ctx, q.d_G, G_aux, (size_t)3 * n_ipw)) || (rc = cuda_check(ctx, cudaMemcpyAsync(q.d_v, d_in, nv * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "copy v")) ||
-        (rc = sync(ctx)))
-        return rc;
+    const bool resized = first || q.nipw != n_ipw;
+    if (resized && !(first && d_in)) {
+        q.set = false;
+        dfree(q.d_VD); dfree(q.d_VB);
+        q.d_VD = nullptr; q.d_VB = nullptr;
+        q.vd_cap = q.vb_cap = 0;
+        if ((rc = place())) return rc;
+    }
+    if ((rc = h2d(ctx, q.d_G, G_aux, (size_t)3 * n_ipw))) return rc;
+    if (!d_in) {
+        if ((rc = upload(q.d_v))) return rc;
+        // (for its other task: the imaginary parts within the tolerance are set to zero)
+        if (ctx->opt.inversion) launch_check_coulomb(q.d_v, naux, 1, d_chk, ctx->stream);
+    } else if (!first) {
+        rc = cuda_check(ctx, cudaMemcpyAsync(q.d_v, d_in, nv * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "copy v");
+        if (rc) return rc;
+    }
+    if ((rc = cuda_check(ctx, cudaGetLastError(), "set_coulomb")) || (rc = sync(ctx))) return rc;
     if (!q.set || q.nipw != n_ipw || q.G.size() != (size_t)3 * n_ipw ||
         (n_ipw > 0 && std::memcmp(q.G.data(), G_aux, sizeof(int) * 3 * n_ipw) != 0))
         ++ctx->struct_epoch;
@@ -533,8 +623,9 @@ void hfx_destroy(hfx_ctx *ctx) {
     dfree(ctx->d_R); dfree(ctx->d_mu); dfree(ctx->d_T); dfree(ctx->d_Tid); dfree(ctx->d_gaunt); dfree(ctx->d_posf);
     dfree(ctx->d_err); dfree(ctx->d_Ex); dfree(ctx->d_radC);
     Scratch *all[] = {&ctx->s_theta, &ctx->s_thpsi, &ctx->s_B,    &ctx->s_zc,   &ctx->s_zs,   &ctx->s_ys,
-                      &ctx->s_y64,   &ctx->s_praw,  &ctx->s_vacc, &ctx->s_pairs, &ctx->s_qd,  &ctx->s_misc,
-                      &ctx->s_ap,    &ctx->s_aexp,  &ctx->s_xexp, &ctx->s_zipw, &ctx->s_cgT, &ctx->s_cgZ};
+                      &ctx->s_y64,   &ctx->s_praw,  &ctx->s_vacc, &ctx->s_pairs, &ctx->s_vin, &ctx->s_misc,
+                      &ctx->s_ap,    &ctx->s_aexp,  &ctx->s_xexp, &ctx->s_zipw, &ctx->s_cgT, &ctx->s_cgZ,
+                      &ctx->s_chk};
     for (Scratch *s : all) dfree(s->p);
     delete ctx;
 }
@@ -720,6 +811,7 @@ int build(hfx_ctx *ctx, const std::vector<int> &kset, int keep, hfx_stats *st) {
     if (keep && ctx->opt.inversion)
         return set_err(ctx, HFX_EUNSUPPORTED, "keep_products: not available with inversion symmetry");
     if ((rc = cuda_check(ctx, cudaSetDevice(ctx->device), "cudaSetDevice"))) return rc;
+    release(ctx->s_vin);
     if ((rc = prepare_coulomb(ctx)) || (rc = prepare_q0(ctx))) return rc;
     return build_run(ctx, kset, keep, st);
 }

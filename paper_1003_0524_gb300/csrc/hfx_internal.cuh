@@ -192,8 +192,9 @@ struct hfx_ctx {
     std::map<std::pair<int, int>, double2 *> zkeep;
 
     // scratch
-    hfx::Scratch s_theta, s_thpsi, s_B, s_zc, s_zs, s_ys, s_y64, s_praw, s_vacc, s_pairs, s_qd,
+    hfx::Scratch s_theta, s_thpsi, s_B, s_zc, s_zs, s_ys, s_y64, s_praw, s_vacc, s_pairs,
         s_misc, s_ap, s_aexp, s_xexp, s_zipw, s_cgT, s_cgZ;
+    hfx::Scratch s_vin, s_chk;   // set_coulomb: a v being checked (until the next build), the check's result
 
     // bumped whenever a plane-wave list, an aux list or a band window changes;
     // host tables built from the structure are reused while it stays the same
