@@ -533,6 +533,7 @@ int hfx_set_coulomb(hfx_ctx *ctx, int iq, int n_ipw, const int *G_aux, const dou
     q.G.assign(G_aux, G_aux + 3 * n_ipw);
     q.nipw = n_ipw;
     q.layout = layout;
+    q.herm = dev == 0.0;
     q.set = true;
     ctx->coulomb_dirty = true;
     ctx->built = false;

@@ -105,6 +105,7 @@ struct QPoint {
     double2 *d_VB = nullptr;     // [n_ch][P-1][P]  mu=0 rows inside their channel
     size_t vd_cap = 0, vb_cap = 0;  // allocated elements of d_VD, d_VB
     int layout = HFX_LAYOUT_DENSE;  // how v was given (dense, or already transformed)
+    bool herm = true;               // v was Hermitian to the last bit
 };
 
 struct Scratch {                 // growable device buffers
@@ -175,6 +176,13 @@ struct hfx_ctx {
     bool coulomb_dirty = true;   // transform must be redone
     bool sparse_used = false;
     bool mod_used = false;       // the Coulomb apply runs on residues (s_ap, s_aexp hold those of U)
+    // FP64 build: apply all of v_t instead of its upper triangle (some v(q) is Hermitian
+    // only within herm_tol: its two triangles hold different numbers)
+    bool full_v() const {
+        bool f = false;
+        for (auto &q : qp) f |= !q.herm;
+        return f && opt.precision == HFX_PREC_FP64;
+    }
     int N0 = 0;                  // mu=0 rows (sparse) or 0 (dense)
     double q0_bracket = 0.0;
     bool q0_valid = false;
@@ -305,7 +313,7 @@ struct ZGemmBatch {         // C = op(A) * B, complex double, K = K1 * K2
 int zgemm64_tile(int M, int N, long long nbatch);   // tile edge launch_zgemm64 takes for these sizes
 void launch_zgemm64(const ZGemmBatch *d_b, int nbatch, int maxM, int maxN, cudaStream_t st);
 void launch_block64(const QDesc *d_q, int nq, const double2 *const *d_VB, const double2 *d_Z, double2 *d_Y,
-                    long long RSc, int nch, int P, int N0, long long maxcols, cudaStream_t st);
+                    long long RSc, int nch, int P, int N0, int full, long long maxcols, cudaStream_t st);
 
 // ------------------------------------------------------------ kernels (tensor-core contraction, k_contract_tc.cu)
 template <typename V>

@@ -106,7 +106,7 @@ int hfx_lapw_transform_all(hfx_ctx *ctx, hfx_stats *st) {
         ZGemmBatch &d = g3[ik];
         d.A = B; d.B = W; d.C = Vg;
         d.M = np; d.N = np; d.K1 = 1; d.K2 = nb;
-        d.sAi = 1; d.sAk1 = 0; d.sAk2 = np; d.sBk1 = 0; d.sBk2 = np; d.sBj = 1; d.sCi = np; d.sCj = 1; d.conjA = 1; d.upper = 0; d.herm = 1;
+        d.sAi = 1; d.sAk1 = 0; d.sAk2 = np; d.sBk1 = 0; d.sBk2 = np; d.sBj = 1; d.sCi = np; d.sCj = 1; d.conjA = 1; d.upper = 0; d.herm = ctx->full_v() ? 0 : 1;
         flops += 8.0 * ((double)nb * np * np + (double)nb * nb * np + (double)np * np * nb);
     }
     if ((rc = scratch_reserve(ctx, ctx->s_lapw_tab, 3 * (size_t)nk * sizeof(ZGemmBatch)))) return rc;

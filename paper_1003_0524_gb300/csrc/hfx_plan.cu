@@ -179,6 +179,7 @@ struct BuildPlan {
     size_t o_A = 0, o_c = 0, o_G = 0, o_Ga = 0, o_npw = 0, o_nb = 0, o_no = 0, o_B = 0, o_T = 0, o_vacc = 0, o_V = 0;
     bool kp = false;                  // the k.p term at q = 0 is added
     bool inv = false;                 // inversion symmetry: packed real bands (Sec. III.D)
+    bool full = false;                // FP64 build: all of v_t is applied
     size_t o_reach = 0;               // T box points that are needed (FP64 build)
     int nreach = 0;
     size_t o_sym = 0;                 // row operations Z' = S^H Z
@@ -245,6 +246,7 @@ uint64_t plan_signature(hfx_ctx *ctx, const std::vector<int> &kset) {
     h.val(ctx->q0_bracket);
     h.val(ctx->sparse_used);
     h.val(ctx->mod_used);
+    h.val(ctx->full_v());
     h.val(ctx->N0);
     for (auto &k : ctx->kp) { h.val(k.d_G); h.val(k.d_c); h.val(k.d_A); h.val(k.nb); h.val(k.no); h.val(k.npw); }
     for (auto &q : ctx->qp) { h.val(q.d_G); h.val(q.d_VD); h.val(q.d_VB); h.val(q.nipw); }
@@ -279,6 +281,7 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         pl.npw_max = std::max(pl.npw_max, k.npw);
     }
     pl.inv = ctx->opt.inversion != 0;
+    pl.full = ctx->full_v();
     pl.RSc = naux_max;
     pl.N0pad = (int)rup(N0, 64);
     pl.Dpad = (int)rup(pl.maxD, 128);
@@ -492,10 +495,10 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
             pl.flops += f * m * n * (nnz + (double)qd.naux * n) + f * m * n * ctx->nlmp * nmt +
                         f * m * n * qd.nipw * hnpw[pr.ikp];
             pl.fl_apply += f * m * n * (double)qd.D * qd.D;
-            // as executed: the upper triangle, over the packed columns
+            // as executed: the upper triangle (or all of v_t), over the packed columns
             // (two real parts of Y' per column with a real v_t)
             const double mc = pr.no, fe = pl.inv ? 4.0 : 8.0;
-            pl.fl_apply_exec += (tc ? fe : 8.0) * mc * n * 0.5 * (double)qd.D * (qd.D + 1);
+            pl.fl_apply_exec += (tc ? fe : 8.0) * mc * n * (pl.full ? (double)qd.D * qd.naux : 0.5 * (double)qd.D * (qd.D + 1));
             pl.fl_zhy += f * m * n * (double)qd.naux * n;
             pl.fl_zipw += f * m * n * (double)qd.nipw * hnpw[pr.ikp];
         }
@@ -606,21 +609,22 @@ int plan_build(hfx_ctx *ctx, const std::vector<int> &kset, BuildPlan &pl) {
         } else {
             std::vector<ZGemmBatch> g1(nq), g2((size_t)npairs * ksplit);
             for (int i = 0; i < nq; ++i) {
-                // the dense-block rows of U: columns [N0, naux) of the rows of v_t
+                // the dense-block rows of U: columns [N0, naux) of the rows of v_t (or all columns)
+                const int k0 = pl.full ? 0 : N0;
                 const QDesc &q = bt.qd[i];
                 ZGemmBatch &b = g1[i];
-                b.A = ctx->qp[q.iq].d_VD + N0;
-                b.B = reinterpret_cast<const double2 *>(Zc) + q.colbase * RSc + N0;
+                b.A = ctx->qp[q.iq].d_VD + k0;
+                b.B = reinterpret_cast<const double2 *>(Zc) + q.colbase * RSc + k0;
                 b.C = Y + q.colbase * RSc + N0;
                 b.M = q.D;
                 b.N = (int)q.ncols;
                 b.K1 = 1;
-                b.K2 = q.D;
+                b.K2 = q.naux - k0;
                 b.sAi = q.naux; b.sAk2 = 1; b.sAk1 = 0;
                 b.sBk2 = 1; b.sBk1 = 0; b.sBj = RSc;
                 b.sCi = 1; b.sCj = RSc;
                 b.conjA = 0;
-                b.upper = 1;
+                b.upper = pl.full ? 0 : 1;
                 b.herm = 0;
                 bt.maxM1 = std::max(bt.maxM1, b.M);
                 bt.maxN1 = std::max(bt.maxN1, b.N);
@@ -859,7 +863,7 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
             launch_zgemm64(reinterpret_cast<const ZGemmBatch *>(tab + bt.o_zg1), nq, bt.maxM1, bt.maxN1, ctx->stream);
             rec(ctx, bt.ev[7]);
             launch_block64(d_qd, nq, reinterpret_cast<const double2 *const *>(tab + bt.o_vb),
-                           reinterpret_cast<const double2 *>(Zc), Yd, RSc, nch, P, N0, bt.maxcols, ctx->stream);
+                           reinterpret_cast<const double2 *>(Zc), Yd, RSc, nch, P, N0, pl.full ? 1 : 0, bt.maxcols, ctx->stream);
             rec(ctx, bt.ev[8]);
             launch_zgemm64(reinterpret_cast<const ZGemmBatch *>(tab + bt.o_zg2), npairs * pl.ksplit, bt.mx2, bt.mx2, ctx->stream);
             rec(ctx, bt.ev[9]);
@@ -869,7 +873,7 @@ int plan_run(hfx_ctx *ctx, BuildPlan &pl, int keep, int fail_wait) {
         launch_reduce_pairs(d_pairs, reinterpret_cast<const int *>(tab + bt.o_kstart),
                             reinterpret_cast<const int *>(tab + bt.o_klp), bt.nklist,
                             reinterpret_cast<const int *>(tab + bt.o_klist), praw, d_praw_off, pl.NB,
-                            tc ? ((pl.inv && gemm2_real_form(pl.NB)) ? 2 : 1) : 0, pl.ksplit,
+                            tc ? ((pl.inv && gemm2_real_form(pl.NB)) ? 2 : 1) : (pl.full ? 3 : 0), pl.ksplit,
                             pl.inv ? 1 : 0, reinterpret_cast<double2 *const *>(tab + pl.o_vacc),
                             reinterpret_cast<const int *>(tab + pl.o_nb),
                             pl.nb_max, ctx->stream);

@@ -2,6 +2,7 @@
 // Y' = U Z (dense block and mu=0 blocks of Fig. 1; U the upper triangle of v_t
 // with half its diagonal, v_t = U + U^H) and the per-pair P' = sum_m Z_m^H Y'_m,
 // whose P' + P'^H is the pair's term of Eq. vec-mat-vec, with DFMA on the CUDA cores.
+// Where v is Hermitian only within a tolerance, all of v_t is applied and Z^H Y is the term.
 #include <algorithm>
 #include <cmath>
 
@@ -113,10 +114,10 @@ int zgemm64_r(int M, int N, long long nbatch) {
 // Y' rows of the mu=0 functions: per channel, the (P-1) x P block of U times the
 // channel's [mu!=0, mu=0...] rows of Z (Fig. 1 on-site blocks): the coupling to the
 // mu!=0 function lies above the diagonal, of the mu=0 functions those from i on count,
-// i itself half.
+// i itself half (full: those of v_t, all of them).
 __global__ void block64_kernel(const QDesc *__restrict__ qd, const double2 *const *__restrict__ VB,
                                const double2 *__restrict__ Z, double2 *__restrict__ Y, long long RSc, int nch, int P,
-                               int N0) {
+                               int N0, int full) {
     const QDesc q = qd[blockIdx.y];
     const double2 *vb = VB[blockIdx.y];
     long long total = q.ncols * N0;
@@ -128,8 +129,8 @@ __global__ void block64_kernel(const QDesc *__restrict__ qd, const double2 *cons
         const double2 *z = Z + col * RSc;
         const double2 *row = vb + ((size_t)ch * (P - 1) + i) * P;
         double2 acc = cmul(row[0], z[N0 + ch]);
-        for (int s = i + 1; s < P; ++s) {
-            const double w = s == i + 1 ? 0.5 : 1.0;
+        for (int s = full ? 1 : i + 1; s < P; ++s) {
+            const double w = !full && s == i + 1 ? 0.5 : 1.0;
             acc = cfma(make_double2(w * row[s].x, w * row[s].y), z[ch * (P - 1) + s - 1], acc);
         }
         Y[col * RSc + u] = acc;
@@ -153,13 +154,13 @@ void launch_zgemm64(const ZGemmBatch *d_b, int nbatch, int maxM, int maxN, cudaS
 }
 
 void launch_block64(const QDesc *d_q, int nq, const double2 *const *d_VB, const double2 *d_Z, double2 *d_Y,
-                    long long RSc, int nch, int P, int N0, long long maxcols, cudaStream_t st) {
+                    long long RSc, int nch, int P, int N0, int full, long long maxcols, cudaStream_t st) {
     if (N0 == 0 || nq == 0) return;
     long long per = maxcols * N0;
     long long g = (per + 255) / 256;
     if (g > 4096) g = 4096;
     dim3 grid((unsigned)g, (unsigned)nq);
-    block64_kernel<<<grid, 256, 0, st>>>(d_q, d_VB, d_Z, d_Y, RSc, nch, P, N0);
+    block64_kernel<<<grid, 256, 0, st>>>(d_q, d_VB, d_Z, d_Y, RSc, nch, P, N0, full);
 }
 
 }  // namespace hfx

@@ -8,7 +8,8 @@ namespace {
 
 // Vacc[k] += sum_{pairs of k in this batch, ascending q} P_pair, where the pair's
 // buffer holds P' = Z^H U Z and P_pair = P' + P'^H (raw_format 0: FP64, 1: the
-// tensor-core tiles, 2: the real tiles of the inversion-symmetric path, Re P' only).
+// tensor-core tiles, 2: the real tiles of the inversion-symmetric path, Re P' only) or
+// P_pair itself (raw_format 3: FP64, all of v_t applied).
 // With real_part (inversion symmetry, two real bands packed per column, Sec.
 // III.D) only the real part is the pair's term; the imaginary part holds the
 // cross products of the two bands and is dropped.
@@ -28,11 +29,12 @@ __global__ void reduce_pairs_kernel(const PairDesc *__restrict__ pairs, const in
         for (int t = p0; t < p1; ++t) {
             int pi = klist_pairs[t];
             const double *P = praw + praw_off[pi];
-            if (raw_format == 0) {
-                // FP64: P' = Z^H U Z in nsplit partial sums over the occupied bands
+            if (raw_format == 0 || raw_format == 3) {
+                // FP64: nsplit partial sums over the occupied bands
                 const double2 *Pc = reinterpret_cast<const double2 *>(P);
                 for (int s = 0; s < nsplit; ++s, Pc += (size_t)nb * nb) {
-                    const double2 v = Pc[(size_t)n * nb + n2], w = Pc[(size_t)n2 * nb + n];
+                    const double2 v = Pc[(size_t)n * nb + n2];
+                    const double2 w = raw_format == 0 ? Pc[(size_t)n2 * nb + n] : make_double2(0.0, 0.0);
                     acc.x += v.x + w.x;
                     if (!real_part) acc.y += v.y - w.y;
                 }
