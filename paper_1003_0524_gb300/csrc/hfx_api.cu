@@ -813,6 +813,9 @@ int build(hfx_ctx *ctx, const std::vector<int> &kset, int keep, hfx_stats *st) {
         return set_err(ctx, HFX_EUNSUPPORTED, "keep_products: not available with inversion symmetry");
     if ((rc = cuda_check(ctx, cudaSetDevice(ctx->device), "cudaSetDevice"))) return rc;
     release(ctx->s_vin);
+    // the working memory of set_radial_functions is kept while it is small (2 MB at lmax 4
+    // and 600 points); 8192 points take 70 MB at lmax 8
+    if (ctx->s_misc.bytes > ((size_t)16 << 20)) release(ctx->s_misc);
     if ((rc = prepare_coulomb(ctx)) || (rc = prepare_q0(ctx))) return rc;
     return build_run(ctx, kset, keep, st);
 }

@@ -30,3 +30,20 @@ def test_functions_are_orthonormal(lmax, Lmax, P, n_r, seed):
         hfx.hfx_destroy(ctx)
     for m in M:
         assert np.abs((m * w * r * r) @ m.T - np.eye(P)).max() <= 2 * n_r * np.finfo(float).eps
+
+
+def test_large_working_memory_is_given_back():
+    """8192 points of lmax 8 need 40 MB; after the next build they are free again, up to
+    the 2 MB granules of an allocation."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    s = S.make_system(dict(S.CONFIGS[0], lmax=8), mesh=(1, 1, 1), nb=2, no=1)
+    r, w, u = S.radial_functions(s.lmax, float(s.rmt[0]), 8192, 3)
+    with hfx.Context(s, sparse="off") as c:
+        c.load_system()
+        c.build_all()
+        free = torch.cuda.mem_get_info()[0]
+        hfx.hfx_set_radial_functions(c.ctx, 0, r, w, u, 1e-4)
+        c.build_all()
+        assert free - torch.cuda.mem_get_info()[0] <= 8 << 20
