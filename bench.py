@@ -61,13 +61,11 @@ def _profiled_traffic(kernel_file: str, profile: str):
     return int(m.group(1))
 
 
-def _apply_kernel(s, st):
+def _apply_kernel(st):
     """The kernel of the dense-block Coulomb apply and its tensor products per real
-    multiply-add: 10 digit products, or, for complex dense blocks of 1664 to 6144 rows,
-    4.5 residue products (18 for a complex one: 9 moduli, 2 real products each)."""
-    n_lm = s.n_atoms * (s.Lmax + 1) ** 2
-    D = max((n_lm if st["sparse_used"] else s.n_mt) + int(g.shape[0]) for g in s.Gaux)
-    return ("mod_gemm_kernel", 4.5) if not s.inversion and 1664 <= D <= 6144 else ("gemm1_kernel", 10.0)
+    multiply-add, a quarter of those of a complex one: 10 digit or 4.5 residue products."""
+    p = st["apply_products"]
+    return "gemm1_kernel" if p == 40 else "mod_gemm_kernel", p / 4.0
 
 
 def _peaks():
@@ -421,7 +419,7 @@ def run_ours(args):
             "zipw": (avg("ms_zipw"), st["flops_zipw"]),
         }
         dom = max(kernels, key=lambda k: kernels[k][0])
-        apply_name, apply_products = _apply_kernel(s, st)
+        apply_name, apply_products = _apply_kernel(st)
         products = {"apply": apply_products, "zhy": 10.0, "zipw": 10.0}
         names = {"apply": apply_name, "zhy": "gemm2_kernel", "zipw": "zipw_tc_kernel"}
         sfx = f"config{args.config}" + ("_inversion" if args.inversion else "")

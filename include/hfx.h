@@ -188,9 +188,14 @@ typedef struct {
     int graph_replayed;       /* 1 if the build was the replay of a captured CUDA graph */
     int tile_nb_zhy;          /* band block of the Z^H Y tiles used */
     int tile_nb_zipw;         /* band block of the interstitial tiles used (0: FP64 build) */
+    int apply_products;       /* tensor products of the dense-block apply per 8 flops of
+                                 flops_apply_exec (a complex multiply-add): 40 (digits),
+                                 18 (residues), 0 (FP64 build) */
     double flops_apply_exec;  /* flops of the dense-block apply as executed: the upper
                                  triangle U of v_t (half diagonal) is applied and
-                                 P' + P'^H added, 8 D (D+1)/2 per column */
+                                 P' + P'^H added, 8 D (D+1)/2 per column; the FP64 build
+                                 of a v that is not Hermitian to the last bit applies all
+                                 of v_t, 8 D N_aux */
 } hfx_stats;
 
 /* ------------------------------------------------------------ entry points */
@@ -258,6 +263,8 @@ HFX_API int hfx_set_kpoint(hfx_ctx *ctx, int ik, int n_bands, int n_occ, int npw
  *                 the next build (after every hfx_set_radial).
  *                 HFX_LAYOUT_TRANSFORMED: v is already v_t (Sec. III.C, Fig. 1) for
  *                 the T of hfx_get_transform; it is used as given.
+ * The sliced build reads the upper triangle of v_t; the FP64 build applies v_t as
+ * given, by its upper triangle where v is Hermitian to the last bit.
  * Errors: HFX_EINVAL (index, size, ld or layout), HFX_ENONFINITE, HFX_ENOTHERM. */
 HFX_API int hfx_set_coulomb(hfx_ctx *ctx, int iq, int n_ipw, const int *G_aux, const double *v, int ld, int layout);
 

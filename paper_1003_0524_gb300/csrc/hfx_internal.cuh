@@ -351,6 +351,7 @@ struct ModSizes {            // of the largest dense block
     size_t col_bytes = 0;    // bytes of the residues of one column of Z or Y'
 };
 bool apply_mod_usable(int maxD);
+int apply_mod_products();    // per complex multiply-add
 ModSizes apply_mod_sizes(int maxD);
 int apply_mod_prepare_u(hfx_ctx *ctx, const double2 *d_VD, __nv_bfloat16 *d_UR, int *d_uexp, int D, int naux, int N0,
                         const ModSizes &z);

@@ -941,6 +941,7 @@ void fill_stats(hfx_ctx *ctx, BuildPlan &pl, hfx_stats *st, bool graph) {
     st->graph_replayed = graph ? 1 : 0;
     st->tile_nb_zhy = pl.NB;
     st->tile_nb_zipw = pl.zipw.NBt;
+    st->apply_products = !pl.tc ? 0 : (pl.mod ? apply_mod_products() : 40);
 }
 
 template <typename R>

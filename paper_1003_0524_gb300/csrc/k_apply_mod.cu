@@ -813,6 +813,8 @@ __global__ void __launch_bounds__(MY_THREADS) mod_y_kernel(const short *__restri
 // than the largest one of the digits (2^-31 of a line's largest element, see above).
 bool apply_mod_usable(int maxD) { return maxD >= 1664 && maxD <= 6144; }
 
+int apply_mod_products() { return NRP; }
+
 ModSizes apply_mod_sizes(int maxD) {
     ModSizes z;
     z.Kp = (maxD + M_KB - 1) / M_KB * M_KB;

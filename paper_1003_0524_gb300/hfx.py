@@ -100,6 +100,7 @@ class hfx_stats(ctypes.Structure):
         ("graph_replayed", ctypes.c_int),
         ("tile_nb_zhy", ctypes.c_int),
         ("tile_nb_zipw", ctypes.c_int),
+        ("apply_products", ctypes.c_int),
         ("flops_apply_exec", ctypes.c_double),
     ]
 
