@@ -467,11 +467,13 @@ __global__ void __launch_bounds__(RO_THREADS) radial_orthonormal_kernel(int n_r,
                 K[a][b] = a == b ? 1.0 / sqrt(s) : s * K[b][b];
             }
     __syncthreads();
+    // (K is close to the unit matrix: its difference from that is added, one rounding)
     for (int i = threadIdx.x; i < n_r; i += RO_THREADS)
         for (int a = 0; a < P; ++a) {
-            double v = ML[(size_t)a * n_r + i];
-            for (int j = 0; j < a; ++j) v = fma(-K[a][j], ML[(size_t)j * n_r + i], v);
-            ML[(size_t)a * n_r + i] = v * K[a][a];
+            const double m = ML[(size_t)a * n_r + i];
+            double c = 0.0;
+            for (int j = 0; j < a; ++j) c = fma(-K[a][j], ML[(size_t)j * n_r + i], c);
+            ML[(size_t)a * n_r + i] = m + fma(m, K[a][a] - 1.0, c * K[a][a]);
         }
 }
 
