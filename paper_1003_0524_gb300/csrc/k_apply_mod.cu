@@ -698,14 +698,7 @@ __device__ __forceinline__ Digits slice_i64(long long F, int x) {
         if (-x > 63) q = 0;
     }
     const unsigned long long neg = (unsigned long long)(F >> 63);
-    const unsigned long long v = (q ^ neg) - neg + 0x808080ULL;
-    const uint32_t vl = (uint32_t)v, vh = (uint32_t)(v >> 32);
-    Digits d;
-    d.s[0] = __float_as_uint(__int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 24)) - 12582912.0f);
-    d.s[1] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7442)) - 8388736.0f);
-    d.s[2] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7441)) - 8388736.0f);
-    d.s[3] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.0f);
-    return d;
+    return digits_of((long long)((q ^ neg) - neg));
 }
 
 __global__ void __launch_bounds__(MY_THREADS) mod_y_kernel(const short *__restrict__ YR, const double2 *__restrict__ Y0,

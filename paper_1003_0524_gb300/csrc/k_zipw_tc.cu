@@ -213,8 +213,7 @@ struct ZParams {
     int td0, nyb, nzb, ly, lz, nblk, nslot;
     float4 *ZI;                   // output plane ZI[g][col] (rows g of the interstitial part, G-major)
     long long NCi;                // row stride of ZI: the columns of the batch
-    int nmt, nk, R, Rpad, nbmax, tlo0, tlo1, tlo2;
-    double rs;                    // Omega^{-1/2}
+    int nk, R, Rpad, tlo0, tlo1, tlo2;
     int *err;
 };
 
@@ -905,13 +904,10 @@ int zipw_tc_run_batch(hfx_ctx *ctx, const ZipwBuild &zb, const ZipwBatch &bt, co
     p.nslot = bt.nslot;
     p.ZI = d_ZI;
     p.NCi = NCi;
-    p.nmt = ctx->nmt;
     p.nk = ctx->nk;
     p.R = zb.R;
     p.Rpad = zb.Rpad;
-    p.nbmax = zb.nb_max;
     p.tlo0 = zb.tlo[0]; p.tlo1 = zb.tlo[1]; p.tlo2 = zb.tlo[2];
-    p.rs = 1.0 / sqrt(ctx->omega);
     p.err = ctx->d_err;
     const int grid = std::min<int>(num_sms(), p.ntiles);
     // the whole opt-in shared memory: the pipeline stages plus a guard region

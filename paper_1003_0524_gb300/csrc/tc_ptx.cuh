@@ -299,25 +299,6 @@ __device__ __forceinline__ int line_exp_bits(unsigned long long b) {
 // a float.  Taking the digits one by one in 64 bits took twice as many and held the
 // slicing of Y at 0.7 of the copy bandwidth (6.6 ms for 30 GB, 4.8 ms now).
 struct Digits { uint32_t s[4]; };
-__device__ __forceinline__ Digits slice4f(double x, int e) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int E = (int)((hi >> 20) & 0x7ffu);
-    // N = m 2^-sh; sh >= 21 because |x| < 2^e; zeros and subnormals give 0
-    const int sh = E ? 1043 + e - E : 64;
-    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-    const int s1 = min(sh, 63);
-    const unsigned long long r = m + ((1ULL << (s1 - 1)) - 1) + ((m >> s1) & 1ULL);
-    const unsigned long long q = sh < 64 ? r >> s1 : 0ULL;
-    const unsigned long long neg = (unsigned long long)((long long)(int)hi >> 63);
-    const unsigned long long v = (q ^ neg) - neg + 0x808080ULL;
-    const uint32_t vl = (uint32_t)v, vh = (uint32_t)(v >> 32);
-    Digits d;
-    d.s[0] = __float_as_uint(__int_as_float(0x4B400000 + (int)__funnelshift_r(vl, vh, 24)) - 12582912.0f);
-    d.s[1] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7442)) - 8388736.0f);
-    d.s[2] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7441)) - 8388736.0f);
-    d.s[3] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.0f);
-    return d;
-}
 // the digits of N, |N| <= 2^32
 __device__ __forceinline__ Digits digits_of(long long N) {
     const unsigned long long v = (unsigned long long)N + 0x808080ULL;
@@ -328,6 +309,18 @@ __device__ __forceinline__ Digits digits_of(long long N) {
     d.s[2] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7441)) - 8388736.0f);
     d.s[3] = __float_as_uint(__uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.0f);
     return d;
+}
+__device__ __forceinline__ Digits slice4f(double x, int e) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int E = (int)((hi >> 20) & 0x7ffu);
+    // N = m 2^-sh; sh >= 21 because |x| < 2^e; zeros and subnormals give 0
+    const int sh = E ? 1043 + e - E : 64;
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    const int s1 = min(sh, 63);
+    const unsigned long long r = m + ((1ULL << (s1 - 1)) - 1) + ((m >> s1) & 1ULL);
+    const unsigned long long q = sh < 64 ? r >> s1 : 0ULL;
+    const unsigned long long neg = (unsigned long long)((long long)(int)hi >> 63);
+    return digits_of((long long)((q ^ neg) - neg));
 }
 // x 2^p as an integer with F fraction bits, truncated (|x| 2^(p + F) < 2^62)
 __device__ __forceinline__ long long f32_fixed(float x, int k) {   // k = p + F
