@@ -113,6 +113,7 @@ __constant__ ModTab kTab = make_tab();
 // 64-bit fraction times a power of two, 2^kFracExp for operands of scale 1
 constexpr double kKappa = mod_product() / 604462909807314587353088.0;
 constexpr int kFracExp = 79 - 64;
+static_assert(kKappa > 1.7387, "2^(2 kHalfBits + 1) exceeds M");
 
 // ------------------------------------------------------------- residues
 __device__ __forceinline__ uint64_t f2_both(float x) { return f2_pack(__float_as_uint(x), __float_as_uint(x)); }
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(MZ_THREADS, 3) mod_z_kernel(const float4 *__re
 // Tile: 256 columns of Z (M) x 256 rows of U (N) of one residue plane, shared by the two
 // CTAs of a cluster (cta_group::2): each loads 128 columns and 128 rows, 64 bytes per
 // cycle and SM at the full MMA rate, where a CTA by itself with 128 x 256 would need 96
-// (10.4 ms against 7.9 on 96000 columns of 2660 functions; the digit products: 16.8).  K from the tile's first row on (U is upper
+// (10.4 ms against 7.9 on 96000 columns of 2660 functions with eight moduli; 9.2 with nine; the digit products: 16.7).  K from the tile's first row on (U is upper
 // triangular); three stages of 128 K values (64 KB; with twice the stages of half the size the
 // issuing thread's waits and commits left the tensor cores idle a third of the time); two
 // accumulators of 256 TMEM columns, so that the drain of one K group of 256 overlaps the
