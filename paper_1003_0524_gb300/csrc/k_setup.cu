@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(256) check_coulomb_kernel(double2 *__restrict_
 // exponential is base * ratio^j * exp(-beta c j^2) with the last factor from a
 // table, and four quotients share one division.  About 10 FP64 operations per
 // vector instead of an exponential, a division and a test per point of the
-// bounding box; the 4x4x4 mesh of a 10.3 bohr cell: 0.59 ms instead of 5.1 to 5.7 ms.
+// bounding box; the 4x4x4 mesh of a 10.3 bohr cell: 0.70 ms a call instead of 5.4 to 6.1.
 constexpr int Q0_SEG = 32, Q0_THREADS = 256;
 struct Q0Lattice {
     double b[9];          // rows b_i / m_i
