@@ -722,11 +722,13 @@ int prepare_coulomb(hfx_ctx *ctx) {
     if (ctx->opt.precision == HFX_PREC_SLICED) {
         int maxD = 0;
         for (auto &q : ctx->qp) maxD = std::max(maxD, ctx->nmt + q.nipw - ctx->N0);
-        if (!ctx->opt.inversion && apply_mod_usable(maxD)) {
+        if (!ctx->opt.inversion && apply_mod_usable(maxD) && ctx->mod_off != ctx->struct_epoch) {
             const ModSizes z = apply_mod_sizes(maxD);
             if ((rc = scratch_reserve(ctx, ctx->s_ap, z.u_elems * ctx->nk * sizeof(__nv_bfloat16))) ||
-                (rc = scratch_reserve(ctx, ctx->s_aexp, (size_t)z.Dp * ctx->nk * sizeof(int))))
+                (rc = scratch_reserve(ctx, ctx->s_aexp, (size_t)z.Dp * ctx->nk * sizeof(int)))) {
+                if (rc == HFX_ENOMEM) ctx->mod_used = true;   // (build takes the digits then)
                 return rc;
+            }
             for (int iq = 0; iq < ctx->nk; ++iq) {
                 const int naux = ctx->nmt + ctx->qp[iq].nipw;
                 if ((rc = apply_mod_prepare_u(ctx, ctx->qp[iq].d_VD, reinterpret_cast<__nv_bfloat16 *>(ctx->s_ap.p) + z.u_elems * iq,
@@ -816,8 +818,24 @@ int build(hfx_ctx *ctx, const std::vector<int> &kset, int keep, hfx_stats *st) {
     // the working memory of set_radial_functions is kept while it is small (2 MB at lmax 4
     // and 600 points); 8192 points take 70 MB at lmax 8
     if (ctx->s_misc.bytes > ((size_t)16 << 20)) release(ctx->s_misc);
-    if ((rc = prepare_coulomb(ctx)) || (rc = prepare_q0(ctx))) return rc;
-    return build_run(ctx, kset, keep, st);
+    auto run = [&]() {
+        int e = prepare_coulomb(ctx);
+        if (!e) e = prepare_q0(ctx);
+        return e ? e : build_run(ctx, kset, keep, st);
+    };
+    rc = run();
+    if (rc == HFX_ENOMEM && ctx->mod_used) {
+        // the residues take 88 bytes per element of a column and 36 per element of U, the
+        // digits 64 and 32: what fits with those only is built with those
+        plan_release(ctx);
+        release(ctx->s_ap);
+        release(ctx->s_aexp);
+        ctx->mod_off = ctx->struct_epoch;
+        ctx->coulomb_dirty = true;
+        ctx->err.clear();
+        rc = run();
+    }
+    return rc;
 }
 
 }  // namespace

@@ -176,6 +176,7 @@ struct hfx_ctx {
     bool coulomb_dirty = true;   // transform must be redone
     bool sparse_used = false;
     bool mod_used = false;       // the Coulomb apply runs on residues (s_ap, s_aexp hold those of U)
+    uint64_t mod_off = ~0ULL;    // the struct_epoch whose builds have no memory for the residues
     // FP64 build: apply all of v_t instead of its upper triangle (some v(q) is Hermitian
     // only within herm_tol: its two triangles hold different numbers)
     bool full_v() const {
